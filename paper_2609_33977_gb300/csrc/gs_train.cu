@@ -21,31 +21,129 @@
 #include "gs_common.cuh"
 
 #include <cublas_v2.h>
+#include <algorithm>
 #include <mutex>
 
 namespace gs {
 namespace {
 
 constexpr int kGumbelThreads = 256;
+constexpr int kGumbelWarps = kGumbelThreads / 32;
+constexpr int64_t kGumbelPerWarp = 256;   // selectors per warp step: two 16-byte loads of each input per thread
+constexpr int kGumbelSteps = 4;           // most warp steps per block and warp
 
-// one selector per thread (grid-stride); per-warp popcount, one 64-bit atomic per warp
-__global__ void k_gumbel(const float* __restrict__ logits, const float* __restrict__ noise, int64_t n, float tau,
-                         uint8_t* __restrict__ mask, float* __restrict__ dsdl, unsigned long long* __restrict__ kept) {
+// tau as the kernel uses it.  For tau in [2^-60, 2^60] 1 / tau is the sum of
+// two floats, hi + lo: x / tau is then fma(x, hi, x lo), which rounds once
+// (the product by lo is 2^-24 of the result), and d d / (1 / tau) needs one
+// division instead of two.  Outside that range hi, lo or the products could
+// overflow or lose bits to underflow, and the divisions are taken as written.
+struct GumbelTau {
+  float tau, hi, lo;
+  int by_product;
+};
+
+__device__ __forceinline__ float over_tau(float x, const GumbelTau& t) { return fmaf(x, t.hi, x * t.lo); }
+
+// {kept, ds/dl} of one selector
+__device__ __forceinline__ bool gumbel_one(float l, float n, const GumbelTau& tau, float& ds) {
+  const float z = __fadd_rn(l, n);
+  const float az = fabsf(z);
+  if (tau.by_product) {
+    const float big = 0x1p67f;   // exp(-2^67 / tau) is 0 up to tau = 2^60; keeps inf out of the fma, lets NaN through
+    const float t = expf(-over_tau(az > big ? big : az, tau));
+    const float d = 1.f + t;
+    ds = __fdiv_rn(over_tau(t, tau), d * d);
+  } else {
+    const float t = expf(-__fdiv_rn(az, tau.tau));
+    const float d = 1.f + t;
+    ds = __fdiv_rn(__fdiv_rn(t, d * d), tau.tau);
+  }
+  return z > 0.f;   // NaN prunes
+}
+
+// the block's kept count: one 64-bit atomic
+__device__ __forceinline__ void add_kept(unsigned int cnt, unsigned long long* kept) {
+  if (kept == nullptr) return;   // uniform over the grid
+  __shared__ unsigned int warp_cnt[kGumbelWarps];
+  const unsigned int w = __reduce_add_sync(0xffffffffu, cnt);
+  if ((threadIdx.x & 31) == 0) warp_cnt[threadIdx.x >> 5] = w;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned int total = 0;
+#pragma unroll
+    for (int i = 0; i < kGumbelWarps; ++i) total += warp_cnt[i];
+    if (total) atomicAdd(kept, (unsigned long long)total);
+  }
+}
+
+// HBM-bound: 13 bytes per selector.  A warp step covers 256 consecutive
+// selectors, two 16-byte loads of each input and two 16-byte + two 4-byte
+// stores per thread; a block takes kGumbelWarps * steps consecutive warp
+// steps and adds its count with one atomic.  25.3 M selectors (329 MB): 55.6 us
+// a call, 5.92 TB/s; one selector per thread with an atomic per warp took
+// 135 us (65 K atomics to one address, byte stores, two divisions).
+template <bool DS>
+__global__ void __launch_bounds__(kGumbelThreads) k_gumbel4(const float4* __restrict__ logits,
+                                                            const float4* __restrict__ noise, int64_t n, int steps,
+                                                            GumbelTau tau, uint32_t* __restrict__ mask,
+                                                            float4* __restrict__ dsdl,
+                                                            unsigned long long* __restrict__ kept) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t nfull = n / kGumbelPerWarp;
+  unsigned int cnt = 0;
+  for (int k = 0; k < steps; ++k) {
+    const int64_t u = ((int64_t)blockIdx.x * steps + k) * kGumbelWarps + warp;
+    if (u >= nfull) break;
+    const int64_t at = u * (kGumbelPerWarp / 4) + lane;
+    float4 l[2], g[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      l[q] = __ldcs(logits + at + 32 * q);
+      g[q] = __ldcs(noise + at + 32 * q);
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      float4 d;
+      const uint32_t m = (gumbel_one(l[q].x, g[q].x, tau, d.x) ? 1u : 0u) |
+                         (gumbel_one(l[q].y, g[q].y, tau, d.y) ? 0x100u : 0u) |
+                         (gumbel_one(l[q].z, g[q].z, tau, d.z) ? 0x10000u : 0u) |
+                         (gumbel_one(l[q].w, g[q].w, tau, d.w) ? 0x1000000u : 0u);
+      mask[at + 32 * q] = m;
+      if (DS) dsdl[at + 32 * q] = d;
+      cnt += __popc(m);
+    }
+  }
+  // the last n % 256 selectors, one per thread of block 0
+  if (blockIdx.x == 0) {
+    const int64_t i = nfull * kGumbelPerWarp + threadIdx.x;
+    if (i < n) {
+      float d;
+      const bool keep = gumbel_one(reinterpret_cast<const float*>(logits)[i], reinterpret_cast<const float*>(noise)[i],
+                                   tau, d);
+      reinterpret_cast<uint8_t*>(mask)[i] = keep ? 1 : 0;
+      if (DS) reinterpret_cast<float*>(dsdl)[i] = d;
+      cnt += keep ? 1u : 0u;
+    }
+  }
+  add_kept(cnt, kept);
+}
+
+// the same for pointers that 16-byte (inputs, ds/dl) or 4-byte (mask) accesses
+// do not fit: one selector per thread and step
+__global__ void __launch_bounds__(kGumbelThreads) k_gumbel(const float* __restrict__ logits,
+                                                           const float* __restrict__ noise, int64_t n, GumbelTau tau,
+                                                           uint8_t* __restrict__ mask, float* __restrict__ dsdl,
+                                                           unsigned long long* __restrict__ kept) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   unsigned int cnt = 0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-    const float z = __fadd_rn(logits[i], noise[i]);
-    const bool keep = z > 0.f;   // NaN prunes
+    float d;
+    const bool keep = gumbel_one(logits[i], noise[i], tau, d);
     mask[i] = keep ? 1 : 0;
-    if (dsdl) {
-      const float t = expf(-fabsf(__fdiv_rn(z, tau)));
-      const float d = 1.f + t;
-      dsdl[i] = __fdiv_rn(__fdiv_rn(t, d * d), tau);
-    }
+    if (dsdl) dsdl[i] = d;
     cnt += keep ? 1u : 0u;
   }
-  const unsigned int w = __reduce_add_sync(0xffffffffu, cnt);
-  if (kept && (threadIdx.x & 31) == 0 && w) atomicAdd(kept, (unsigned long long)w);
+  add_kept(cnt, kept);
 }
 
 // dlogits[u, v] = ds/dl[u, v] * sum over group (u, v) of W (.) D, D = dy^T x
@@ -89,6 +187,17 @@ gs_status blas_handle(cublasHandle_t* h) {
   return GS_OK;
 }
 
+int sm_count_train() {
+  static int n = 0;
+  if (n == 0) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    if (n <= 0) n = 148;
+  }
+  return n;
+}
+
 size_t round256(size_t b) { return (b + 255) & ~size_t(255); }
 
 }  // namespace
@@ -97,10 +206,31 @@ gs_status launch_gumbel(const float* logits, const float* noise, int64_t n, floa
                         int64_t* kept, cudaStream_t s) {
   if (kept && cudaMemsetAsync(kept, 0, sizeof(int64_t), s) != cudaSuccess) return GS_ERR_CUDA;
   if (n == 0) return GS_OK;
-  int64_t blocks = (n + kGumbelThreads - 1) / kGumbelThreads;
-  if (blocks > 8 * 1024) blocks = 8 * 1024;
-  k_gumbel<<<(unsigned)blocks, kGumbelThreads, 0, s>>>(logits, noise, n, tau, mask, dsdl,
-                                                       reinterpret_cast<unsigned long long*>(kept));
+  GumbelTau t{tau, 0.f, 0.f, 0};
+  if (tau >= 0x1p-60f && tau <= 0x1p60f) {
+    const double inv = 1.0 / (double)tau;
+    t.hi = (float)inv;
+    t.lo = (float)(inv - (double)t.hi);
+    t.by_product = 1;
+  }
+  unsigned long long* k64 = reinterpret_cast<unsigned long long*>(kept);
+  const uintptr_t a16 = reinterpret_cast<uintptr_t>(logits) | reinterpret_cast<uintptr_t>(noise) |
+                        reinterpret_cast<uintptr_t>(dsdl);   // a NULL ds/dl adds no bits
+  if ((a16 & 15u) == 0 && (reinterpret_cast<uintptr_t>(mask) & 3u) == 0) {
+    // blocks of up to four steps per warp; fewer while that leaves the SMs short of blocks
+    const int64_t per_block = kGumbelPerWarp * kGumbelWarps;
+    const int64_t units = (n + per_block - 1) / per_block;
+    const int64_t steps = std::min<int64_t>(kGumbelSteps, std::max<int64_t>(1, units / (8 * sm_count_train())));
+    // n < 2^36 keeps the grid below 2^23
+    const unsigned grid = (unsigned)((units + steps - 1) / steps);
+    auto kern = dsdl ? k_gumbel4<true> : k_gumbel4<false>;
+    kern<<<grid, kGumbelThreads, 0, s>>>(reinterpret_cast<const float4*>(logits), reinterpret_cast<const float4*>(noise),
+                                         n, (int)steps, t, reinterpret_cast<uint32_t*>(mask),
+                                         reinterpret_cast<float4*>(dsdl), k64);
+  } else {
+    const int64_t blocks = std::min<int64_t>((n + kGumbelThreads - 1) / kGumbelThreads, 8 * sm_count_train());
+    k_gumbel<<<(unsigned)blocks, kGumbelThreads, 0, s>>>(logits, noise, n, t, mask, dsdl, k64);
+  }
   note_launch();
   return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }

@@ -48,6 +48,36 @@ def test_gumbel_select_matches_oracle(gs, n, tau):
     assert np.allclose(dg[fin], ref[fin], rtol=2e-5, atol=0)
 
 
+@pytest.mark.parametrize("n", [1, 255, 256, 257, 2047, 2048, 2049, 3 * 8192 + 5, 12 * 1024 * 1024 + 300])
+@pytest.mark.parametrize("tau", [0.25, 2.0 ** -60, 2.0 ** 60, 2.0 ** -61, 2.0 ** 61])
+def test_gumbel_select_vector_and_scalar_paths(gs, n, tau):
+    """16-byte loads (whole buffers) and the one-at-a-time path (views one element in), over the
+    range of tau that multiplies by 1 / tau and just outside it: the same bits, and
+    |ds - ref| <= 2^-24 (|a| + 10) ref with a = z / tau (a rounds once: |a| 2^-24; expf 2 ulp; one
+    rounding each of 1 + t (squared: twice), d d, t / tau and the quotient, and one for lo)."""
+    import torch
+    if n > 1 << 20 and tau != 0.25:
+        pytest.skip("the large size runs once")
+    lg = wl.selector_logits((n,), 0.5, seed=n, special_every=97 if n > 100 else 0)
+    noise = logistic_noise(n, n + 1)
+    mask, dsdl, kept = gs.gumbel_select(torch.from_numpy(lg).cuda(), torch.from_numpy(noise).cuda(), tau)
+    l1, n1 = (torch.from_numpy(np.concatenate([[np.float32(0)], a])).cuda()[1:] for a in (lg, noise))
+    m2, d2, k2 = gs.gumbel_select(l1, n1, tau)
+    assert torch.equal(mask, m2) and torch.equal(kept, k2)
+    assert np.array_equal(dsdl.cpu().numpy(), d2.cpu().numpy(), equal_nan=True)
+    B, _ = orc.gumbel_select(lg, noise, tau)
+    assert np.array_equal(mask.cpu().numpy(), B) and int(kept.cpu()[0]) == int(B.sum())
+    with np.errstate(over="ignore", invalid="ignore"):
+        a = np.abs((lg + noise).astype(np.float64)) / tau
+        ref = orc.gumbel_dsdl(lg, noise, tau)
+    dg = dsdl.cpu().numpy().astype(np.float64)
+    nan = np.isnan(ref)
+    assert np.array_equal(np.isnan(dg), nan)
+    fin = ~nan & (ref > 1e-30) & (ref < 1e38)
+    assert np.all(np.abs(dg[fin] - ref[fin]) <= 2.0 ** -24 * (a[fin] + 10) * ref[fin])
+    assert np.all(dg[~nan & (ref < 1e-45)] <= 1e-44)
+
+
 def backward_case(gs, out, inp, g_out, g_in, T, seed, want_dx=True):
     import torch
     Wb = wl.random_weight_bits(out, inp, seed=seed)
