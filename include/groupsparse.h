@@ -250,7 +250,15 @@ gs_status gs_packed_export(const gs_packed* p, int64_t* offsets_host, int32_t* r
 gs_status gs_pack_index_noalloc(const uint8_t* mask_dev, int64_t out, int64_t in, int64_t* offsets_dev,
                                 int32_t* win_off16_dev, uint16_t* kmask16_dev, void* stream);
 
-/* Releases the handle and its device buffers (NULL is a no-op). */
+/*
+ * Releases the handle (NULL is a no-op).  Work already queued with the handle
+ * completes.  If the handle was used on gs_pack's stream only, and not inside a
+ * graph capture, its device buffers are kept for the next gs_pack on that
+ * stream, at most 1/128 of the device's memory in all; they return to the
+ * device when that is exceeded, when they stay unused, or when an allocation of
+ * the library finds the device out of memory.  Otherwise they are freed at
+ * once (cudaFree, which waits for the device).
+ */
 void gs_free(gs_packed* p);
 
 /* Static description of a status code. */

@@ -34,28 +34,19 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 
 void free_buffers(gs_packed* p) {
   if (!p) return;
-  int cur = -1;
-  cudaGetDevice(&cur);
-  if (cur != p->device) cudaSetDevice(p->device);
-  if (p->offsets) cudaFree(p->offsets);
-  if (p->row_idx) cudaFree(p->row_idx);
-  if (p->tiles) cudaFree(p->tiles);
-  if (p->win_off16) cudaFree(p->win_off16);
-  if (p->kmask16) cudaFree(p->kmask16);
   decode_release(p);
-  sq_release(p);
-  if (cur >= 0 && cur != p->device) cudaSetDevice(cur);
-  p->offsets = nullptr;
-  p->row_idx = nullptr;
-  p->tiles = nullptr;
-  p->win_off16 = nullptr;
-  p->kmask16 = nullptr;
+  // Work of several streams, or of graph replays, is not ordered before what
+  // the pack stream runs next: those buffers are freed.
+  PoolTag tag = p->tag;
+  if (__atomic_load_n(&p->shared, __ATOMIC_ACQUIRE)) tag.valid = false;
+  for (int i = 0; i < p->nbufs; ++i) pool_give(p->bufs[i], tag);
+  p->nbufs = 0;
 }
 
-gs_status dev_alloc(void** ptr, size_t bytes, size_t* total) {
+gs_status dev_alloc(gs_packed* p, void** ptr, size_t bytes, size_t* total) {
   *ptr = nullptr;
   if (bytes == 0) return GS_OK;
-  const gs_status st = lib_malloc(ptr, bytes);
+  const gs_status st = handle_malloc(p, ptr, bytes);
   if (st == GS_OK) *total += bytes;
   return st;
 }
@@ -89,12 +80,104 @@ void note_launch(int64_t n) { g_launches.fetch_add(n, std::memory_order_relaxed)
 
 uint64_t timeout_epoch() { return g_timeout_epoch.load(std::memory_order_acquire); }
 
-gs_status lib_malloc(void** ptr, size_t bytes) {
-  *ptr = nullptr;
+// true: the armed allocation fails as if the device were full
+static bool fail_this_alloc() {
   int64_t n = g_fail_alloc_in.load(std::memory_order_relaxed);
   while (n > 0 && !g_fail_alloc_in.compare_exchange_weak(n, n - 1)) {
   }
-  if (n == 1) return GS_ERR_OOM;   // the armed allocation fails as if the device were full
+  return n == 1;
+}
+
+gs_status handle_malloc(gs_packed* p, void** ptr, size_t bytes) {
+  *ptr = nullptr;
+  if (p->nbufs >= kHandleBufs) return GS_ERR_OOM;
+  if (fail_this_alloc()) return GS_ERR_OOM;
+  const cudaError_t e = pool_take(&p->bufs[p->nbufs], bytes, p->tag);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    return GS_ERR_OOM;
+  }
+  if (e != cudaSuccess) return GS_ERR_CUDA;
+  *ptr = p->bufs[p->nbufs++].ptr;
+  return GS_OK;
+}
+
+void handle_free(gs_packed* p, const void* ptr) {
+  for (int i = 0; i < p->nbufs; ++i) {
+    if (p->bufs[i].ptr != ptr) continue;
+    pool_give(p->bufs[i], p->tag);
+    p->bufs[i] = p->bufs[--p->nbufs];
+    return;
+  }
+}
+
+void handles_used(const gs_packed* const* ps, int n, cudaStream_t s) {
+  int captured = -1;   // asked at most once per call
+  for (int i = 0; i < n; ++i) {
+    int32_t* shared = const_cast<int32_t*>(&ps[i]->shared);   // the one mutable field besides the scratch table
+    if (__atomic_load_n(shared, __ATOMIC_RELAXED)) continue;
+    if (captured < 0) {
+      cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+      const cudaError_t e = cudaStreamIsCapturing(s, &st);
+      if (e != cudaSuccess) cudaGetLastError();   // the launch that follows reports what is wrong with s
+      captured = e != cudaSuccess || st != cudaStreamCaptureStatusNone ? 1 : 0;
+    }
+    if (captured || static_cast<void*>(s) != ps[i]->pack_stream) __atomic_store_n(shared, 1, __ATOMIC_RELEASE);
+  }
+}
+
+void handle_on_stream(gs_packed* p, cudaStream_t s) {
+  p->pack_stream = static_cast<void*>(s);
+  p->tag = pool_tag(p->device, s);
+  // one address, another stream in every thread: no identity to compare
+  if (s == cudaStreamPerThread) p->tag.valid = false;
+}
+
+// Pinned words that gs_pack reads kept counts through (a pageable copy is
+// staged, with a wait of its own): one page, a bit per word in use.
+class PinnedWord {
+ public:
+  PinnedWord() {
+    std::lock_guard<std::mutex> lk(mu());
+    if (!page() && !tried()) {
+      tried() = true;
+      if (cudaHostAlloc(reinterpret_cast<void**>(&page()), 64 * sizeof(int64_t), cudaHostAllocPortable) != cudaSuccess) {
+        cudaGetLastError();
+        page() = nullptr;
+      }
+    }
+    if (!page() || used() == ~uint64_t(0)) return;   // the caller's own word then
+    bit_ = __builtin_ctzll(~used());
+    used() |= uint64_t(1) << bit_;
+  }
+  ~PinnedWord() {
+    if (bit_ < 0) return;
+    std::lock_guard<std::mutex> lk(mu());
+    used() &= ~(uint64_t(1) << bit_);
+  }
+  int64_t* get() { return bit_ < 0 ? &own_ : page() + bit_; }
+
+ private:
+  static std::mutex& mu() { static std::mutex* m = new std::mutex; return *m; }
+  static int64_t*& page() { static int64_t* p = nullptr; return p; }
+  static bool& tried() { static bool t = false; return t; }
+  static uint64_t& used() { static uint64_t u = 0; return u; }
+  int bit_ = -1;
+  int64_t own_ = 0;
+};
+
+gs_status read_kept(gs_packed* p, const int64_t* kept_dev, cudaStream_t s) {
+  PinnedWord w;
+  if (cudaMemcpyAsync(w.get(), kept_dev, sizeof(int64_t), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess)
+    return GS_ERR_CUDA;
+  p->kept = *w.get();
+  return GS_OK;
+}
+
+gs_status lib_malloc(void** ptr, size_t bytes) {
+  *ptr = nullptr;
+  if (fail_this_alloc()) return GS_ERR_OOM;
   const cudaError_t e = cudaMalloc(ptr, bytes);
   if (e == cudaErrorMemoryAllocation) {
     cudaGetLastError();
@@ -151,34 +234,26 @@ static gs_status pack_rows(const void* W_dev, const uint8_t* mask_dev, int64_t o
   p->g_out = 1;
   p->g_in = kw;
   p->Gout = (int32_t)out;
+  handle_on_stream(p, s);
 
   size_t total = 0;
   int32_t* cnt = nullptr;
   gs_status st = GS_OK;
   const size_t E = (size_t)p->G * (size_t)p->nw16;
-  if ((st = dev_alloc((void**)&p->offsets, sizeof(int64_t) * (size_t)(G + 1), &total)) != GS_OK) goto fail;
-  if ((st = dev_alloc((void**)&p->win_off16, sizeof(int32_t) * (size_t)p->G * (size_t)(p->nw16 + 1), &total)) !=
+  if ((st = dev_alloc(p, (void**)&p->offsets, sizeof(int64_t) * (size_t)(G + 1), &total)) != GS_OK) goto fail;
+  if ((st = dev_alloc(p, (void**)&p->win_off16, sizeof(int32_t) * (size_t)p->G * (size_t)(p->nw16 + 1), &total)) !=
       GS_OK)
     goto fail;
-  if ((st = dev_alloc((void**)&p->kmask16, sizeof(uint16_t) * E, &total)) != GS_OK) goto fail;
+  if ((st = dev_alloc(p, (void**)&p->kmask16, sizeof(uint16_t) * E, &total)) != GS_OK) goto fail;
   {
     size_t scratch = 0;
-    if ((st = dev_alloc((void**)&cnt, sizeof(int32_t) * E, &scratch)) != GS_OK) goto fail;
+    if ((st = dev_alloc(p, (void**)&cnt, sizeof(int32_t) * E, &scratch)) != GS_OK) goto fail;
   }
   if ((st = launch_pack_count_scan(mask_dev, p, s, cnt)) != GS_OK) goto fail;
-  {
-    int64_t kept = 0;
-    if (cudaMemcpyAsync(&kept, p->offsets + G, sizeof(int64_t), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess) {
-      st = GS_ERR_CUDA;
-      goto fail;
-    }
-    p->kept = kept;
-  }
-  cudaFree(cnt);
-  cnt = nullptr;
-  if ((st = dev_alloc((void**)&p->row_idx, sizeof(int32_t) * (size_t)p->kept, &total)) != GS_OK) goto fail;
-  if ((st = dev_alloc((void**)&p->tiles, 2 * (size_t)kw * (size_t)p->kept, &total)) != GS_OK) goto fail;
+  if ((st = read_kept(p, p->offsets + G, s)) != GS_OK) goto fail;
+  handle_free(p, cnt);
+  if ((st = dev_alloc(p, (void**)&p->row_idx, sizeof(int32_t) * (size_t)p->kept, &total)) != GS_OK) goto fail;
+  if ((st = dev_alloc(p, (void**)&p->tiles, 2 * (size_t)kw * (size_t)p->kept, &total)) != GS_OK) goto fail;
   p->device_bytes = total;
   if ((st = launch_pack_compact(W_dev, p, s)) != GS_OK) goto fail;
   if ((st = decode_prepare(p, s)) != GS_OK) goto fail;
@@ -187,7 +262,6 @@ static gs_status pack_rows(const void* W_dev, const uint8_t* mask_dev, int64_t o
   return GS_OK;
 
 fail:
-  if (cnt) cudaFree(cnt);
   free_buffers(p);
   delete p;
   return st;
@@ -230,6 +304,7 @@ gs_status gs_pack_groups(const void* W_dev, const uint8_t* mask_dev, int64_t out
   p->G = (int32_t)Gin;
   p->Gout = (int32_t)Gout;
   p->nwin = (int32_t)((out + 127) / 128);
+  handle_on_stream(p, static_cast<cudaStream_t>(stream));
   const gs_status st = sq_pack(W_dev, mask_dev, p, static_cast<cudaStream_t>(stream));
   if (st != GS_OK) {
     free_buffers(p);
@@ -257,6 +332,7 @@ static gs_status linear_impl(const void* x_dev, const gs_packed* p, int64_t T, v
   if (!x_dev || !y_dev) return GS_ERR_INVALID_ARG;
   if (!aligned16(x_dev) || !aligned16(y_dev)) return GS_ERR_INVALID_ARG;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  handles_used(&p, 1, s);
   if (is_square(p)) return sq_linear_batched(&x_dev, &p, 1, T, &y_dev, s);   // one kernel family for every T
   if (algo == GS_ALGO_AUTO) {
     // the same per-layer choice as gs_linear_batched makes
@@ -303,6 +379,7 @@ gs_status gs_linear_batched(int32_t n, const void* const* xs_dev, const gs_packe
   }
   if (T == 0) return GS_OK;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  handles_used(ps, n, s);
   {
     // square-group layers take their own launches; the 1 x 256 layers continue below
     std::vector<const void*> xq;
@@ -402,6 +479,7 @@ gs_status gs_select_groups(const float* logits_dev, int64_t n, uint8_t* mask_dev
 
 gs_status gs_unpack(const gs_packed* p, void* W_hat_dev, void* stream) {
   if (check_handle(p) != GS_OK || !W_hat_dev || !aligned16(W_hat_dev)) return GS_ERR_INVALID_ARG;
+  handles_used(&p, 1, static_cast<cudaStream_t>(stream));
   if (is_square(p)) return sq_unpack(p, W_hat_dev, static_cast<cudaStream_t>(stream));
   return launch_unpack(p, W_hat_dev, static_cast<cudaStream_t>(stream));
 }
@@ -541,6 +619,7 @@ gs_status gs_masked_linear_backward(const void* x_dev, const void* W_dev, const 
     return GS_ERR_INVALID_ARG;
   if (p->out > INT32_MAX || p->in > INT32_MAX) return GS_ERR_UNSUPPORTED;
   if (workspace_bytes < backward_workspace_bytes(p, dx_dev != nullptr)) return GS_ERR_INVALID_ARG;
+  handles_used(&p, 1, static_cast<cudaStream_t>(stream));
   return launch_backward(x_dev, W_dev, p, dy_dev, T, dsdl_dev, dlogits_dev, dx_dev, workspace_dev,
                          static_cast<cudaStream_t>(stream));
 }

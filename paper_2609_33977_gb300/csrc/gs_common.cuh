@@ -30,11 +30,31 @@ struct DecSlot {
   uint64_t epoch;     // timeout epoch at which the counters were last known clean
 };
 
+// One device buffer of the library (allocated bytes) and where an idle one may
+// be used again: on that device, for work queued on that stream.
+struct PoolBuf {
+  void* ptr;
+  size_t bytes;
+};
+struct PoolTag {
+  int device;
+  bool valid;                      // false: no stream identity, buffers go back to cudaFree
+  unsigned long long stream_id;    // cudaStreamGetId
+};
+constexpr int kHandleBufs = 12;
+
 }  // namespace gs
 
 // Library-owned packed weight.  All arrays live on `device`.
 struct gs_packed {
   int device;
+  // the handle's buffers (every array below, and the split scratch of the pack
+  // stream) and the identity of the stream gs_pack queued its work on
+  gs::PoolBuf bufs[gs::kHandleBufs];
+  int32_t nbufs;
+  gs::PoolTag tag;
+  void* pack_stream;   // cudaStream_t, compared only
+  int32_t shared;      // atomic: used on another stream than gs_pack's, or captured into a graph
   int64_t out, in;
   int32_t G;          // in / 256
   int32_t nw16;       // ceil(out / 16)
@@ -103,6 +123,20 @@ uint64_t timeout_epoch();
 // Every device allocation of the library goes through here (so that a test can
 // make the n-th one fail); OOM on cudaErrorMemoryAllocation, else CUDA.
 gs_status lib_malloc(void** ptr, size_t bytes);
+// the same for a buffer that handle p owns: it comes from the pool and returns
+// there, or to cudaFree, with the handle
+gs_status handle_malloc(gs_packed* p, void** ptr, size_t bytes);
+void handle_free(gs_packed* p, const void* ptr);   // one of them, before the handle goes
+// fills in the pack stream and its identity
+void handle_on_stream(gs_packed* p, cudaStream_t s);
+// notes that work using the handles is queued on s (before every call's first launch)
+void handles_used(const gs_packed* const* ps, int n, cudaStream_t s);
+// waits for s and reads the kept-group count into p->kept
+gs_status read_kept(gs_packed* p, const int64_t* kept_dev, cudaStream_t s);
+// pool.cu: idle device buffers of released handles
+PoolTag pool_tag(int device, cudaStream_t s);
+cudaError_t pool_take(PoolBuf* buf, size_t bytes, const PoolTag& tag);
+void pool_give(const PoolBuf& buf, const PoolTag& tag);   // an invalid tag: cudaFree
 // Test hook: limit of a wait on the never-set word to inject into the next
 // launch of a kernel family (GS_ALGO_DECODE / GS_ALGO_PREFILL /
 // GS_ALGO_PREFILL_DENSE); 0 = none.
@@ -132,7 +166,7 @@ gs_status launch_select(const float* logits, int64_t n, uint8_t* mask, int64_t* 
 
 // decode.cu
 gs_status decode_prepare(gs_packed* p, cudaStream_t s);   // allocates + builds the decode metadata
-void decode_release(gs_packed* p);
+void decode_release(gs_packed* p);   // the split scratch of streams other than the pack stream
 // split scratch of handle p for stream s (made on first use; re-zeroed after a timeout)
 gs_status decode_slot(const gs_packed* p, cudaStream_t s, const DecSlot** slot);
 gs_status launch_decode(const gs_packed* const* ps, const void* const* xs, void* const* ys, int n, int T,
@@ -158,7 +192,6 @@ gs_status sq_pack(const void* W, const uint8_t* mask, gs_packed* p, cudaStream_t
 gs_status sq_unpack(const gs_packed* p, void* W_hat, cudaStream_t s);
 gs_status sq_linear_batched(const void* const* xs, const gs_packed* const* ps, int n, int64_t T, void* const* ys,
                             cudaStream_t s);
-void sq_release(gs_packed* p);
 // sq_decode.cu: square groups, T <= sq_decode_max_tokens(): layers ps[idx[0..n)] (same g, kept > 0, n <= 8)
 int sq_decode_max_tokens();
 gs_status sq_decode_batched(const void* const* xs, const gs_packed* const* ps, const int* idx, int n, int T,

@@ -641,6 +641,11 @@ cudaError_t launch_nt(const DecParams<MB>& P, int grid, cudaStream_t s) {
 
 int decode_max_tokens() { return kMaxT; }
 
+namespace {
+size_t slot_ws_floats(const gs_packed* p) { return (size_t)p->nblk64 * p->dec_nsplit_max * kDW * kPartFloats; }
+size_t slot_counters(const gs_packed* p) { return (size_t)p->nblk64 * kDW + 2; }   // + {unit ticket, finished CTAs}
+}  // namespace
+
 gs_status decode_prepare(gs_packed* p, cudaStream_t s) {
   p->nblk64 = (int32_t)((p->out + kRows - 1) / kRows);
   // Chunks per unit: a block's chunks are split into the whole number of
@@ -657,16 +662,22 @@ gs_status decode_prepare(gs_packed* p, cudaStream_t s) {
   p->dec_cpu_fine = std::max(1, cpu / 4);
   p->dec_nsplit_max = (p->G + p->dec_cpu_fine - 1) / p->dec_cpu_fine;
   const size_t nmeta = (size_t)p->nblk64 * (size_t)p->G;
-  {
-    const gs_status am = lib_malloc(reinterpret_cast<void**>(&p->dmeta), nmeta * sizeof(int4));
-    if (am != GS_OK) return am;
-  }
-  p->device_bytes += nmeta * sizeof(int4);
-  // the split scratch of gs_pack's stream is made now (gs_linear on that
-  // stream then never allocates); other streams get theirs on first use
-  const DecSlot* slot = nullptr;
-  const gs_status st = decode_slot(p, s, &slot);
+  gs_status st = handle_malloc(p, reinterpret_cast<void**>(&p->dmeta), nmeta * sizeof(int4));
   if (st != GS_OK) return st;
+  p->device_bytes += nmeta * sizeof(int4);
+  // The split scratch of gs_pack's stream (slot 0) is made now, so gs_linear on
+  // that stream never allocates; other streams get theirs on first use.  It is
+  // zeroed on that stream: its buffer may be one that earlier work there still uses.
+  DecSlot slot{};
+  slot.stream = static_cast<void*>(s);
+  slot.epoch = timeout_epoch();
+  const size_t nws = slot_ws_floats(p), ncnt = slot_counters(p);
+  if ((st = handle_malloc(p, reinterpret_cast<void**>(&slot.ws), nws * sizeof(float))) != GS_OK) return st;
+  if ((st = handle_malloc(p, reinterpret_cast<void**>(&slot.cnt), ncnt * sizeof(int32_t))) != GS_OK) return st;
+  if (cudaMemsetAsync(slot.cnt, 0, ncnt * sizeof(int32_t), s) != cudaSuccess) return GS_ERR_CUDA;
+  p->dec_slot[0] = slot;
+  p->dec_nslots = 1;
+  p->device_bytes += nws * sizeof(float) + ncnt * sizeof(int32_t);
   const int64_t n = (int64_t)nmeta;
   k_pack_decode_meta<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(p->win_off16, p->kmask16, p->G, p->nw16, p->nblk64,
                                                            p->dmeta);
@@ -675,21 +686,24 @@ gs_status decode_prepare(gs_packed* p, cudaStream_t s) {
 }
 
 void decode_release(gs_packed* p) {
-  if (p->dmeta) cudaFree(p->dmeta);
-  p->dmeta = nullptr;
   std::lock_guard<std::mutex> lk(g_slot_mu);
-  for (int i = 0; i < p->dec_nslots; ++i) {
-    if (p->dec_slot[i].ws) cudaFree(p->dec_slot[i].ws);
-    if (p->dec_slot[i].cnt) cudaFree(p->dec_slot[i].cnt);
-    p->dec_slot[i] = DecSlot{};
+  if (p->dec_nslots > 1) {
+    int cur = -1;
+    cudaGetDevice(&cur);
+    if (cur != p->device) cudaSetDevice(p->device);
+    for (int i = 1; i < p->dec_nslots; ++i) {   // slot 0 is among the handle's buffers
+      cudaFree(p->dec_slot[i].ws);
+      cudaFree(p->dec_slot[i].cnt);
+    }
+    if (cur >= 0 && cur != p->device) cudaSetDevice(cur);
   }
+  for (int i = 0; i < p->dec_nslots; ++i) p->dec_slot[i] = DecSlot{};
   p->dec_nslots = 0;
 }
 
 gs_status decode_slot(const gs_packed* pc, cudaStream_t s, const DecSlot** out) {
   gs_packed* p = const_cast<gs_packed*>(pc);   // the slot table is the only mutable part of a handle
-  const size_t nws = (size_t)p->nblk64 * p->dec_nsplit_max * kDW * kPartFloats;
-  const size_t ncnt = (size_t)p->nblk64 * kDW + 2;   // + {unit ticket, finished CTAs}
+  const size_t nws = slot_ws_floats(p), ncnt = slot_counters(p);
   const uint64_t epoch = timeout_epoch();
   std::lock_guard<std::mutex> lk(g_slot_mu);
   DecSlot* slot = nullptr;

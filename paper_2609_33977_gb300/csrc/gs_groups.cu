@@ -619,7 +619,7 @@ gs_status sq_pack(const void* W, const uint8_t* mask, gs_packed* p, cudaStream_t
       *ptr = nullptr;
       return GS_OK;
     }
-    const gs_status st = lib_malloc(ptr, bytes);
+    const gs_status st = handle_malloc(p, ptr, bytes);
     if (st == GS_OK) total += bytes;
     return st;
   };
@@ -628,20 +628,16 @@ gs_status sq_pack(const void* W, const uint8_t* mask, gs_packed* p, cudaStream_t
   if ((st = alloc((void**)&p->offsets, sizeof(int64_t) * (size_t)(Gin + 1))) != GS_OK) return st;
   if ((st = alloc((void**)&p->gwoff, sizeof(int32_t) * (size_t)(Gin * (nwin + 1)))) != GS_OK) return st;
   if ((st = alloc((void**)&p->gwmask, (size_t)E)) != GS_OK) return st;
-  if ((st = lib_malloc((void**)&cnt, sizeof(int32_t) * (size_t)E)) != GS_OK) return st;
+  if ((st = handle_malloc(p, (void**)&cnt, sizeof(int32_t) * (size_t)E)) != GS_OK) return st;
   k_sq_count<<<(unsigned)((E + 255) / 256), 256, 0, s>>>(mask, (int32_t)Gout, (int32_t)Gin, R, (int32_t)nwin,
                                                          p->gwmask, cnt);
   note_launch();
   st = cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
   if (st == GS_OK) st = launch_scan_counts(cnt, (int32_t)Gin, (int32_t)nwin, p->gwoff, p->offsets, s);
-  int64_t kept = 0;
-  if (st == GS_OK && (cudaMemcpyAsync(&kept, p->offsets + Gin, sizeof(int64_t), cudaMemcpyDeviceToHost, s) !=
-                          cudaSuccess ||
-                      cudaStreamSynchronize(s) != cudaSuccess))
-    st = GS_ERR_CUDA;
-  cudaFree(cnt);
+  if (st == GS_OK) st = read_kept(p, p->offsets + Gin, s);
   if (st != GS_OK) return st;
-  p->kept = kept;
+  handle_free(p, cnt);
+  const int64_t kept = p->kept;
   const size_t tile_elems = (size_t)g * (size_t)g;
   if ((st = alloc((void**)&p->row_idx, sizeof(int32_t) * (size_t)kept)) != GS_OK) return st;
   if ((st = alloc((void**)&p->tiles, 2 * tile_elems * (size_t)kept)) != GS_OK) return st;
@@ -690,15 +686,6 @@ gs_status sq_unpack(const gs_packed* p, void* W_hat, cudaStream_t s) {
       static_cast<uint16_t*>(W_hat));
   note_launch();
   return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
-}
-
-void sq_release(gs_packed* p) {
-  if (p->gwoff) cudaFree(p->gwoff);
-  if (p->gwmask) cudaFree(p->gwmask);
-  if (p->gtidx) cudaFree(p->gtidx);
-  p->gwoff = nullptr;
-  p->gwmask = nullptr;
-  p->gtidx = nullptr;
 }
 
 gs_status sq_linear_batched(const void* const* xs, const gs_packed* const* ps, int n, int64_t T, void* const* ys,
