@@ -57,8 +57,8 @@ constexpr uint32_t kSqTmemCols = kSqAccBufs * kSqWin;
 constexpr int kSqEpiWarps = 4;
 constexpr int kSqThreads = (2 + kSqEpiWarps) * 32;
 constexpr int kSqMaxLayers = 8;
-constexpr int kSqDenseMaxG = 64;          // above the decode regime, g <= this takes the zero-filled kernel (7B block, T = 2048: 64x64 525 vs 476 TFLOP/s)
-constexpr int kSqDecodeMaxTokensZf = 32;  // decode regime of the layers the zero-filled kernel takes
+constexpr int kSqDenseMaxG = 64;          // above the decode regime, g <= this takes the zero-filled kernel (7B block, T = 2048: 64x64 1030 vs 476 TFLOP/s)
+constexpr int kSqDecodeMaxTokensZf = 16;  // decode regime of the layers the zero-filled kernel takes
 constexpr int kSqMaxMaps = 8;             // W slice heights g, 2g, ..., R g (R <= 8)
 constexpr uint64_t kSqWaitLimitNs = 2000000000ull;
 constexpr uint64_t kSqDrainLimitNs = 200000000ull;
@@ -714,10 +714,11 @@ gs_status sq_linear_batched(const void* const* xs, const gs_packed* const* ps, i
     // gives each layer what a single call gives it):
     //  - decode regime: the tile-streaming kernel, one launch per 16 tokens.  Its
     //    time grows with the 16-token blocks while the tensor-core kernels' stays
-    //    flat up to 128 tokens.  Over the five LLaMA-2 7B / 13B projection shapes
-    //    at d = 0.5 the zero-filled-window kernel (layers whose input is whole
-    //    128-column items, g <= 64) takes 1.3-1.5x its time at 32 tokens,
-    //    0.90-1.03x at 48 and 0.37-0.43x at 128; the square tensor-core kernel
+    //    flat up to 128 tokens.  For layers whose input is whole 128-column items,
+    //    g <= 64, the zero-filled-window kernel is ahead from the second launch on
+    //    (us per block at T = 16 / 32, decode against zero-filled: 7B 16x16 52 / 100
+    //    against 67 / 67, 64x64 41 / 81 against 48 / 48, Qwen2.5-7B 32x32 52 / 103
+    //    against 86 / 86); the square tensor-core kernel
     //    (the other layers) breaks even at 128 / 64 / 32 / 16 tokens for
     //    g = 16 / 32 / 64 / 128;
     //  - above it, the zero-filled-window kernel where it applies (dense-layer

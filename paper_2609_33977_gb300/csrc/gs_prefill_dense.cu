@@ -1,39 +1,40 @@
-// Prefill-regime group-sparse linear with zero-filled windows (1 x 256 and
-// 1 x 128 groups, Eq. 1), for layers whose kept fraction is high enough that
-// multiplying the pruned rows by zero costs less than gathering the kept ones.
+// Prefill-regime group-sparse linear with zero-filled windows (1 x 256, 1 x 128
+// and square groups, Eq. 1): the tensor work is that of the dense layer, and only
+// kept weights move.
 //
-// A unit of work is 256 tokens x a window of 256 output rows, owned by a
-// cluster of two CTAs: CTA r holds tokens 128 r .. 128 r + 127 and window rows
-// 128 r .. 128 r + 127.  For every chunk with a kept row in the window and every
-// 64-wide k slab of it, the producer warps place the window's rows in shared
-// memory at their row positions (a 16-byte cp.async per piece from the packed
-// tiles for a kept row; zeros for a pruned row), next to one TMA box of the
-// tokens' x slab, and the leader issues M = 256, N = 256 cta_group::2 MMAs that
-// accumulate the whole unit in TMEM.  Nothing is gathered or scattered: the
-// accumulator is read once per unit.  Packed weights are read from memory once
-// per unit (pruned groups move no bytes); the tensor work is that of the dense
-// window, i.e. 1 / density times the kept work.
+// A unit of work is a window of 256 output rows x a tile of N <= 256 tokens,
+// owned by a cluster of two CTAs: CTA r holds window rows 128 r .. 128 r + 127
+// and tokens r N / 2 .. of the tile.  The weights are the MMA's A operand and
+// live in tensor memory, where lane = output row, so a kept row reaches its row
+// position with one tcgen05.st by the lane that owns it and a pruned row is a
+// register full of zeros:
+//   packed tiles --TMA box--> shared (the half window's kept rows, compact)
+//     --ld.shared by kept lanes--> registers --tcgen05.st--> TMEM A slot.
+// x is the B operand (TMA, 128-byte swizzle).  Per 128-deep K stage the leader
+// issues eight M = 256 x N x 16 cta_group::2 MMAs; D^T (rows x tokens, fp32)
+// stays in TMEM for the whole unit.
 //
-// Roles (one CTA per SM, units persistent over the pairs): warps 0..3
-// producers (warp-cooperative 16-byte cp.async of the window's rows, zero-filled
-// for pruned rows), warp 4 TMEM allocator + single-thread MMA issuer (leader),
-// warps 5..8 epilogue, warp 9 and warps 11.. forwarders (stage pairs taken in
-// turn), warp 10 x producer (TMA).  W slots
-// and x slots are two rings: the W ring (ten 16 KB slots) runs deeper than
-// the x ring (four), because a W slot's round trip (copies landing,
-// fences, arrival at the leader) is about three times a TMA's.  Two
-// consecutive stages share one readiness barrier (both forwarders, both CTAs'
-// x bytes) and one completion barrier: the single MMA-issuing thread spends
-// most of a stage on its own instructions (about 40 ns per MMA, 50 per commit
-// and 60 per wait), so one wait and one commit per stage pair (eight MMAs)
-// instead of two of each per stage took the 13824 x 5120 layer from 1120 to
-// ~1220 dense-equivalent TFLOP/s (1 x 256) and 1 x 128 groups from 0.283 to
-// 0.232 ms; a second forwarder (the fences of one batch take about a
-// microsecond, which one forwarder could no longer hide) then took it to 1440.  Every item therefore has an even number of stages (square groups
-// use 128-column items, two slabs with their own tile lookups).  Producers never wait for their own copies: each thread's copies
-// of a stage signal a local barrier (cp.async.mbarrier.arrive), and the
-// forwarder, once all have landed, fences them to the async proxy and arrives
-// on the leader's full barrier.  Every wait is bounded.
+// Why this split.  Shared memory receives x (N / 2 x 256 B a stage) and the kept
+// rows only, and nothing is written there by threads, so no generic-to-async
+// proxy fence lies between the weights and the tensor cores.  (With the rows
+// placed in shared memory by cp.async, as zero-filled B operands, the copies'
+// fences and the second operand's bytes held a 7B block at T = 2048 to 547 us,
+// 1.52 PFLOP/s dense-equivalent; now 405 us, 2.05 PFLOP/s, at the chip's power limit.)
+//
+// What bounds it.  At N = 256 the tensor cores.  At small N the chain of hand-offs
+// of a stage (copy -> converters -> leader -> commit), about 0.45 us a stage of 128
+// k: 13B block at T = 32 / 128 in 71 / 76 us (4.5 TB/s of kept weights at T = 32).
+// The roles that issue MMAs and copies walk their stages with the whole warp and
+// issue from one elected lane: inside a one-lane branch an MMA cost 70 cycles of
+// issue and a copy 220 to 400 (13B block at T = 128: 92 us).
+//
+// Roles (one CTA per SM, units persistent over the pairs): warp 0 x copies,
+// warp 1 W copies, warp 2 TMEM allocator + MMA issuer (leader), warps 4..11
+// converters (TMEM lane quarter warp & 3; two sets of four warps take the stages
+// in turn), warps 12..19 epilogue (lane quarter warp & 3, half of the tokens
+// each).  The epilogue packs its columns to bf16 in registers and hands D back
+// before it stores, so a single D buffer costs the next unit only that read;
+// tiles of up to 64 tokens have two.  Every wait is bounded.
 #include "gs_common.cuh"
 #include "gs_sm100.cuh"
 
@@ -47,57 +48,58 @@ namespace gs {
 namespace {
 using namespace sm100;
 
-constexpr int kDM = 128;                          // tokens per CTA (TMEM lanes); a pair covers 256
-constexpr int kDW = 256;                          // output rows per window (N of each MMA)
-constexpr int kDHalf = kDW / 2;                   // window rows each CTA holds
-constexpr int kDSlabK = 64;                       // k per stage (one 128-byte swizzle row)
-constexpr int kDXBytes = kDM * kDSlabK * 2;       // 16 KB of x per stage
-constexpr int kDWBytes = kDHalf * kDSlabK * 2;    // 16 KB of W rows per stage
-// Two rings: W slots (the long round trip: copies landing, forwarder fences,
-// arrival at the leader) run deeper than x slots (TMA); with single stages 9 / 3
-// measured ahead of 8 / 4, 7 / 5 and 10 / 2; with stage pairs both counts are
-// even and the shared memory (224 KB) is used up.
-constexpr int kDWStages = 10;                    // 160 KB
-constexpr int kDXStages = 4;                     // 64 KB
-constexpr int kDSuper = kDWStages / 2;          // pairs of consecutive stages share their barriers
-constexpr int kDXRing = kDXStages * kDXBytes;     // 64 KB at offset 0
-constexpr int kDWRing = kDWStages * kDWBytes;     // 128 KB after it
-constexpr int kDProdWarps = 4;                   // warps that copy W rows
-constexpr int kDMmaWarp = kDProdWarps;
-constexpr int kDEpiWarp0 = kDProdWarps + 1;
-constexpr int kDEpiWarps = 4;
-constexpr int kDFwdWarp = kDEpiWarp0 + kDEpiWarps;
-constexpr int kDXWarp = kDFwdWarp + 1;            // x TMA producer
-constexpr int kDNumFwd = 2;                       // forwarders: warp kDFwdWarp, then kDXWarp + 1, ...
-constexpr int kDThreads = (kDXWarp + kDNumFwd) * 32;
-constexpr int kDAccBufs = 2;
-constexpr uint32_t kDTmemCols = kDAccBufs * kDW;  // 512
+constexpr int kDW = 256;                          // output rows per window (M of each MMA)
+constexpr int kDHalf = kDW / 2;                   // window rows each CTA holds (TMEM lanes)
+constexpr int kDN = 256;                          // most tokens per tile (N of each MMA)
+constexpr int kDStageK = 128;                     // k per stage: two 64-wide slabs
+constexpr int kDWBytes = kDHalf * kDStageK * 2;   // 32 KB of kept rows per stage at most
+constexpr int kDMaxXSlots = 8;                    // x slots (shared), at most
+constexpr int kDWSeq = 16;                        // W stages in flight, at most
+constexpr int kDConvWarp0 = 4, kDConvSets = 2, kDConvWarps = 4 * kDConvSets;   // a set per stage, in turn
+constexpr int kDEpiWarp0 = kDConvWarp0 + kDConvWarps, kDEpiWarps = 8;
+constexpr int kDThreads = (kDEpiWarp0 + kDEpiWarps) * 32;
+constexpr int kDMmaWarp = 2;
+constexpr uint32_t kDTmemCols = 512;              // D first, then the A slots of 64 columns each
 constexpr int kDMaxLayers = 8;
+constexpr int kDWMaps = 8;                        // W box heights: 16, 32, ..., 128 rows (square: g, 2g, ..., 128)
 constexpr uint64_t kDWaitLimitNs = 2000000000ull;
 constexpr uint64_t kDDrainLimitNs = 200000000ull;
-constexpr int kDIbufBytes = 1024;                // per-warp chunk lists of d_items
-constexpr int kDSmem = kDXRing + kDWRing + kDIbufBytes + 1024;
-static_assert(kDHalf % (kDProdWarps * 32) == 0, "producer warps split the CTA's window rows evenly");
-static_assert(kDSmem <= 227 * 1024, "shared memory budget");
-static_assert(kDWBytes % 1024 == 0 && kDXBytes % 1024 == 0, "slots keep 1024-byte alignment");
+// Shared memory: x slots of the tile's own size first, the rest is a byte ring
+// for the kept rows, whose stages vary with the density: what is in flight is
+// bytes that move, not slots sized for a full window.
+constexpr int kDRing = 224 * 1024;
+constexpr int kDSmem = kDRing + 1024;
+static_assert(kDSmem <= 226 * 1024, "shared memory budget");
+// x slots of a tile of n tokens (both CTAs): eight where the tile is small
+// (short MMAs: the copies' round trip is what they wait for), four of 32 KB at n = 256
+__host__ __device__ constexpr int d_x_slots(int n) { return n <= kDN / 2 ? kDMaxXSlots : kDMaxXSlots / 2; }
+// TMEM columns of D (n <= 64: two buffers), and the A slots the rest holds: a slot's
+// round trip (both CTAs' converters, the leader, the commit) is about 1.4 us, which
+// four slots hide at n = 256 (0.5 us of MMA a stage) and six about halve at small n
+__host__ __device__ constexpr uint32_t d_d_cols(int n) { return n <= kDN / 2 ? kDN / 2 : kDN; }
+__host__ __device__ constexpr uint32_t d_a_slots(int n) { return (512 - d_d_cols(n)) / (kDStageK / 2); }
+// A W stage that would straddle the ring's end starts over at 0: with every
+// earlier stage released that asks for at most twice the largest stage.
+static_assert(kDRing - d_x_slots(kDN) * (kDN / 2) * kDStageK * 2 >= 2 * kDWBytes &&
+              kDRing - d_x_slots(kDN / 2) * (kDN / 4) * kDStageK * 2 >= 2 * kDWBytes, "two largest W stages fit the ring");
 
 struct DLayer {
-  CUtensorMap xmap;          // x as (64, T, in/64) slabs, box 64 x 128 x 1
-  const uint16_t* tiles;     // 1 x KW: [kept][KW]; square g x g: [kept][g][g]
-  const int32_t* win_off16;  // 1 x KW: [G][nw16 + 1]
-  const uint16_t* kmask16;   // 1 x KW: [G][nw16]
-  const int32_t* gtidx;      // square: [out / g][in / g] packed tile of each group, -1 if pruned
+  CUtensorMap xmap;          // x as (64, T, in/64) slabs, box 64 x N/2 x 2
+  CUtensorMap wmap[kDWMaps]; // kept rows: 1 x KW slabs (box 64 x 16(h+1) x 2), square g x g (box g x g(h+1))
+  const uint16_t* tiles;     // packed weights (square groups of 16 and 32 copy from here)
+  const int32_t* win_off;    // 1 x KW: [G][nw16 + 1]; square: gwoff [in / g][nwin + 1]
+  const void* kmask;         // 1 x KW: uint16 [G][nw16]; square: uint8 [in / g][nwin]
   uint16_t* y;
-  int32_t out, G, nw16, n_m, tile_begin;   // G: chunks of KW columns (square: 64-column slabs)
-  int32_t Gin;               // square: in / g
+  int32_t out, G, nw, n_m, tile_begin;   // G: chunks of KW columns (square: of 128); nw: 16-row (square: 128-row) windows
 };
 struct DParams {
   DLayer L[kDMaxLayers];
-  int32_t n_layers, T, n_tiles;
+  int32_t n_layers, T, N, n_tiles;
   int* err;
   uint64_t inject_ns;   // test hook: CTA pair 0 first waits this long on a word nothing sets (0 = off)
   TileList tl;          // which pair takes which units
 };
+static_assert(sizeof(DParams) <= 32764, "kernel parameter limit");
 
 __device__ __forceinline__ int d_layer_of(const DParams& P, int t) {
   int l = 0;
@@ -105,87 +107,191 @@ __device__ __forceinline__ int d_layer_of(const DParams& P, int t) {
   return l;
 }
 
-// 16-byte copy global -> shared; src_bytes < 16 fills the rest with zeros (0: reads nothing)
-__device__ __forceinline__ void cp_async16_zfill(uint32_t dst, const void* src, uint32_t src_bytes) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
+// true in one lane of a converged warp (the same one each time)
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(r));
+  return r != 0;
 }
-// arrive on a local mbarrier once all of this thread's earlier cp.async copies have landed
-// (without raising its expected count: the barrier counts the arriving threads)
-__device__ __forceinline__ void cp_async_arrive_noinc(uint64_t* bar) {
-  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+// D (M = 256: this CTA's 128 lanes and the peer's) (+)= A (TMEM, the same lanes
+// and columns in both CTAs) * B^T (N rows, half in each CTA's shared memory)
+__device__ __forceinline__ void mma_bf16_ts_pair(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
+                                                 uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
 }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-__device__ __forceinline__ void fence_acq_rel_cluster() { asm volatile("fence.acq_rel.cluster;" ::: "memory"); }
-__device__ __forceinline__ void fence_proxy_async_cta() {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+__device__ __forceinline__ void tmem_st_x32(uint32_t taddr, const uint32_t (&v)[32]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,"
+      "%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};" ::"r"(taddr),
+      "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]),
+      "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]), "r"(v[16]), "r"(v[17]), "r"(v[18]),
+      "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]), "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]),
+      "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31])
+      : "memory");
 }
-
-// Chunks c0 .. c0 + 31 with at least one kept row in window w, in order, into
-// buf (square groups: every 128-column item)
-template <int SQ>
-__device__ __forceinline__ int d_items(const DLayer& L, int w, int c0, int lane, int16_t* buf) {
-  const int c = c0 + lane;
-  __syncwarp();   // every lane is done reading the previous batch
-  bool ne = false;
-  if (c < L.G) {
-    if constexpr (SQ > 0) {
-      ne = true;
-    } else {
-      const int32_t* wo = L.win_off16 + (int64_t)c * (L.nw16 + 1);
-      const int lo = w * (kDW / kWin16), hi = min(lo + kDW / kWin16, L.nw16);
-      ne = wo[hi] > wo[lo];
-    }
-  }
-  const uint32_t ballot = __ballot_sync(0xffffffffu, ne);
-  if (ne) buf[__popc(ballot & ((1u << lane) - 1u))] = (int16_t)c;
-  __syncwarp();
-  return __popc(ballot);
+__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
+      "l"(src), "r"(bytes), "r"(smem_u32(bar))
+      : "memory");
 }
-
+__device__ __forceinline__ uint4 lds128(uint32_t saddr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(saddr) : "memory");
+  return v;
+}
 __device__ __forceinline__ uint32_t d_pack_bf16x2(float lo, float hi) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-// KW: chunk width (1 x KW groups; 128 for square groups: items of two slabs);
-// SQ: 0, or g for square g x g groups
+// Whether item c of window w has MMAs: 1 x KW chunks with a kept row in the
+// window (square groups: every 128-column item)
+template <int SQ>
+__device__ __forceinline__ bool d_nonempty(const DLayer& L, int w, int c) {
+  if (c >= L.G) return false;
+  if constexpr (SQ > 0) return true;
+  const int32_t* wo = L.win_off + (int64_t)c * (L.nw + 1);
+  const int lo = w * (kDW / kWin16), hi = min(lo + kDW / kWin16, L.nw);
+  return wo[hi] > wo[lo];
+}
+// this lane's share of the number of items of window w (summed over the warp later)
+template <int SQ>
+__device__ __forceinline__ int d_count_part(const DLayer& L, int w, int lane) {
+  int n = 0;
+  for (int c = lane; c < L.G; c += 32) n += d_nonempty<SQ>(L, w, c) ? 1 : 0;
+  return n;
+}
+
+__device__ __forceinline__ bool d_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* err) {
+  return mbar_wait_bounded(bar, parity, abort_flag, err, kDWaitLimitNs, kDevErrTimeout);
+}
+__device__ __forceinline__ bool d_wait_cluster(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* err) {
+  return mbar_wait_bounded_cluster(bar, parity, abort_flag, err, kDWaitLimitNs, kDevErrTimeout);
+}
+// the same for a whole warp
+__device__ __forceinline__ bool d_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* err) {
+  return __all_sync(0xffffffffu, d_wait(bar, parity, abort_flag, err));
+}
+
+// Walks a pair's units in batches of 32 items.  Lane l of a warp looks after
+// item c0 + l of the batch; what it loads for the next batch is in flight while
+// the warp works through this one.  (Loaded an item ahead instead, the lookups
+// queue behind the copies in flight: 1.0 us a stage instead of 0.5.)
+template <int SQ>
+struct DWalk {
+  const DParams* P;
+  int pair, n_pairs, ku, u, c0, w, m;
+  const DLayer* L;
+  __device__ __forceinline__ void unit() {
+    u = owner_tile(P->tl, P->n_tiles, pair, n_pairs, ku);
+    c0 = 0;
+    if (u < 0) return;
+    L = &P->L[d_layer_of(*P, u)];
+    const int lt = u - L->tile_begin;
+    m = lt % L->n_m;
+    w = lt / L->n_m;
+  }
+  __device__ __forceinline__ DWalk(const DParams& p, int pr, int n) : P(&p), pair(pr), n_pairs(n), ku(0) { unit(); }
+  __device__ __forceinline__ bool valid() const { return u >= 0; }
+  __device__ __forceinline__ void next() {
+    c0 += 32;
+    if (c0 >= L->G) {
+      ++ku;
+      unit();
+    }
+  }
+};
+// kept rows of a 1 x KW item: first packed row of the window's two halves and the end
+struct DRows {
+  int a, b, c;
+};
+template <int SQ>
+__device__ __forceinline__ DRows d_rows(const DWalk<SQ>& W, int lane) {
+  DRows r = {0, 0, 0};
+  const int c = W.c0 + lane;
+  if (W.valid() && c < W.L->G) {
+    const int nw = W.L->nw, lo = W.w * (kDW / kWin16);
+    const int32_t* wo = W.L->win_off + (int64_t)c * (nw + 1);
+    r.a = wo[lo];
+    r.b = wo[min(lo + kDHalf / kWin16, nw)];
+    r.c = wo[min(lo + kDW / kWin16, nw)];
+  }
+  return r;
+}
+// kept block rows of a square item's column blocks in 128-row window win, R bits each
+template <int SQ>
+__device__ __forceinline__ uint64_t d_blocks(const DWalk<SQ>& W, int win, int lane) {
+  constexpr int kB = SQ > 0 ? kDStageK / SQ : 1, kR = SQ > 0 ? kDHalf / SQ : 1;
+  uint64_t v = 0;
+  const int c = W.c0 + lane;
+  if (W.valid() && c < W.L->G && win < W.L->nw) {
+    const uint8_t* km = static_cast<const uint8_t*>(W.L->kmask) + (int64_t)c * kB * W.L->nw + win;
+#pragma unroll
+    for (int b = 0; b < kB; ++b) v |= (uint64_t)km[(int64_t)b * W.L->nw] << (b * kR);
+  }
+  return v;
+}
+// items of the batch that have MMAs (square groups: every item)
+template <int SQ>
+__device__ __forceinline__ uint32_t d_batch(const DWalk<SQ>& W, const DRows& r, int lane) {
+  if constexpr (SQ > 0) return __ballot_sync(0xffffffffu, W.c0 + lane < W.L->G);
+  return __ballot_sync(0xffffffffu, r.c > r.a);
+}
+
+// KW: item width (1 x KW groups; square groups: 128-column items); SQ: 0, or g
+// for square g x g groups
 template <int KW, int SQ>
 __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_constant__ DParams P) {
-  constexpr int kSlabs = KW / kDSlabK;   // stages per chunk
-  static_assert(kSlabs % 2 == 0 && kDWStages % 2 == 0 && kDXStages % 2 == 0, "stages go in pairs");
+  constexpr int kStPer = KW / kDStageK;                   // stages per item
+  constexpr int kRowK = SQ > 0 ? (SQ < 64 ? SQ : 64) : 64;   // columns of one kept-row piece in shared memory
+  constexpr int kSub = 64 / kRowK;                        // row pieces per 64-wide slab
+  constexpr int kPieces = kRowK / 8;                      // 16-byte pieces per row piece
+  constexpr int kBlk = 2 * kSub;                          // row pieces (square: column blocks) per stage
+  constexpr int kR = SQ > 0 ? kDHalf / SQ : 1;            // square: block rows per half window
+  static_assert(SQ == 0 || KW == kDStageK, "square items are one stage");
   extern __shared__ uint8_t d_smem_raw[];
-  // Stage k uses W slot k % kDWStages and x slot k % kDXStages; one barrier of
-  // each kind per W slot, so the MMA thread waits once and commits once a stage.
-  __shared__ __align__(8) uint64_t full_bar[kDSuper];       // leader: both forwarders + both CTAs' x bytes, two stages
-  __shared__ __align__(8) uint64_t done_bar[kDSuper];       // the two stages' MMAs completed (both CTAs)
-  __shared__ __align__(8) uint64_t wfull_bar[kDWStages];    // local: this CTA's producer threads' copies
-  __shared__ __align__(8) uint64_t afull_bar[kDAccBufs];
-  __shared__ __align__(8) uint64_t aempty_bar[kDAccBufs];
+  __shared__ __align__(8) uint64_t full_bar[kDMaxXSlots];  // leader: both CTAs' converters + both CTAs' x bytes
+  __shared__ __align__(8) uint64_t done_bar[kDMaxXSlots];  // the stage's MMAs completed (both CTAs)
+  __shared__ __align__(8) uint64_t wfull_bar[kDWSeq];      // local: W bytes landed
+  __shared__ __align__(8) uint64_t wempty_bar[kDWSeq];     // local: the converters have read them
+  __shared__ uint32_t w_end[kDWSeq];                       // virtual end of each W stage in the ring (W copy warp)
+  __shared__ int32_t w_start[32][SQ > 0 ? kBlk : 1];       // the batch's items: first packed row (square: tile) ...
+  __shared__ __align__(8) uint64_t w_n[32];                // ... and kept rows (square: kept block rows, d_blocks)
+  __shared__ __align__(8) uint64_t afull_bar[2];          // D complete (both CTAs)
+  __shared__ __align__(8) uint64_t aempty_bar[2];         // leader: D read by both CTAs' epilogues
   __shared__ __align__(8) uint64_t drain_bar;
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_s;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(d_smem_raw) + 1023) & ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();   // 0: leader (issues the pair's MMAs)
-  // chunk lists of d_items (producers, MMA issuer, x producer, forwarders)
-  const int ib_slot = warp <= kDMmaWarp ? warp : warp == kDFwdWarp ? kDMmaWarp + 1 : warp >= kDXWarp ? warp - kDXWarp + kDMmaWarp + 2 : 0;
-  int16_t* ibuf = reinterpret_cast<int16_t*>(smem + kDXRing + kDWRing) + ib_slot * 32;
-  static_assert((kDMmaWarp + 2 + kDNumFwd) * 32 * 2 <= kDIbufBytes, "chunk lists fit");
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kDSuper; ++s) {
-      mbar_init(&full_bar[s], 2 * (2 + 1));   // per stage: both CTAs' forwarders + the leader's expect-tx
+    for (int s = 0; s < kDMaxXSlots; ++s) {
+      mbar_init(&full_bar[s], 2 * 4 + 1);
       mbar_init(&done_bar[s], 1);
     }
-    for (int s = 0; s < kDWStages; ++s) mbar_init(&wfull_bar[s], kDProdWarps * 32);
-    for (int b = 0; b < kDAccBufs; ++b) {
+    for (int s = 0; s < kDWSeq; ++s) {
+      mbar_init(&wfull_bar[s], 1);
+      mbar_init(&wempty_bar[s], 4);
+    }
+    for (int b = 0; b < 2; ++b) {
       mbar_init(&afull_bar[b], 1);
       mbar_init(&aempty_bar[b], 2 * kDEpiWarps);
     }
     mbar_init(&drain_bar, 1);
     abort_s = 0;
     fence_mbar_init();
-    for (int l = 0; l < P.n_layers; ++l) prefetch_tmap(&P.L[l].xmap);
   }
   if (warp == kDMmaWarp) {
     tmem_alloc_pair(&tmem_base_s, kDTmemCols);
@@ -194,10 +300,22 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
   tc_fence_before();
   cluster_sync_all();
   tc_fence_after();
+  // Programmatic dependent launch: a launch that follows may take over SMs as
+  // they fall free; this one copies weights (which only packing writes) at once
+  // and waits for the one before it where x is read and y written.
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const uint32_t tmem = tmem_base_s;
   volatile int* abort_flag = &abort_s;
   const int n_tiles = P.n_tiles;
   const int pair = (int)(blockIdx.x >> 1), n_pairs = (int)(gridDim.x >> 1);
+  const int Nh = P.N / 2;                          // tokens of a tile each CTA loads
+  const uint32_t xs_n = (uint32_t)d_x_slots(P.N);  // x slots; full / done barriers in use
+  const uint32_t xs_bytes = (uint32_t)Nh * (kDStageK * 2);
+  const uint32_t w_ring = (uint32_t)kDRing - xs_n * xs_bytes;   // bytes of the W ring
+  uint8_t* wsmem = smem + xs_n * xs_bytes;
+  const uint32_t n_buf = P.N <= kDN / 4 ? 2u : 1u; // D buffers
+  const uint32_t t_a = d_d_cols(P.N);              // first column of the A slots
+  const uint32_t a_n = d_a_slots(P.N);
 
   if (P.inject_ns != 0 && pair == 0) {
     // test hook: before any copy or MMA is issued, a bounded wait on a word
@@ -221,340 +339,438 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
 
   if (injected_abort) {
     // nothing was issued: go straight to the TMEM release
-  } else if (warp < kDProdWarps) {
-    // ------------------------------------------------------------ producers
-    // Warp v copies window rows v * kRows .. + kRows - 1 of this CTA's half,
-    // warp-cooperatively: copy i moves rows v * kRows + 4 i .. + 3, eight
-    // lanes per 128-byte row, so each instruction reads four whole lines.
-    // Lane l looks up the packed positions of rows v * kRows + 32 q + l.
-    constexpr int kRows = kDHalf / kDProdWarps;   // rows per producer warp
-    constexpr int kOwn = kRows / 32;              // rows whose metadata a lane loads
-    constexpr int kCopies = kRows / 4;            // 16-byte copies per lane per stage
-    uint32_t stage = 0, phase = 0;
+  } else if (warp == 0) {
+    // ------------------------------------------------------------ x copies
+    // Stage k's box goes to slot k % xs_n once stage k - xs_n is done, and
+    // completes on the leader's full barrier.
+    uint32_t s = 0, ph = 1u;
     bool ok = true;
-    for (int ku = 0, u; ok && (u = owner_tile(P.tl, n_tiles, pair, n_pairs, ku)) >= 0; ++ku) {
-      const DLayer& L = P.L[d_layer_of(P, u)];
-      const int w = (u - L.tile_begin) / L.n_m;
-      const int j = lane & 7;   // 16-byte piece of a row this lane copies
-      // 1 x KW: metadata of this lane's rows in chunk c, the window's kept mask
-      // and first packed row (two independent loads, issued one item ahead of use)
-      auto load_meta = [&](int c, uint32_t (&km)[kOwn], int (&wo)[kOwn]) {
-#pragma unroll
-        for (int q = 0; q < kOwn; ++q) {
-          const int h = (int)rank * kDHalf + warp * kRows + 32 * q + lane;   // row within the window
-          const int b16 = min(w * (kDW / kWin16) + (h >> 4), L.nw16 - 1);
-          km[q] = L.kmask16[(int64_t)c * L.nw16 + b16];
-          wo[q] = L.win_off16[(int64_t)c * (L.nw16 + 1) + b16];
-        }
-      };
-      // square: packed tile of each piece this lane copies in each slab of item c
-      // (its row's block row, its columns' block column), loaded one item ahead
-      constexpr int kTS = SQ > 0 ? kSlabs : 1;   // slabs with their own tile lookups
-      // a warp's 32 rows lie in one block row (g >= 32) or two (g = 16): one
-      // lookup per block row and slab; copy i uses block row kU * i / kCopies
-      constexpr int kU = SQ == 16 ? 2 : 1;
-      auto load_tiles = [&](int c, int (&tv)[kTS][kU]) {
-#pragma unroll
-        for (int sl = 0; sl < kTS; ++sl)
-#pragma unroll
-          for (int q = 0; q < kU; ++q) {
-            const int row = w * kDW + (int)rank * kDHalf + warp * kRows + 16 * q;   // first row of the block row part
-            const int k = c * KW + sl * kDSlabK + 8 * j;
-            tv[sl][q] = row < L.out ? L.gtidx[(int64_t)(row / (SQ > 0 ? SQ : 1)) * L.Gin + k / (SQ > 0 ? SQ : 1)] : -1;
+    asm volatile("griddepcontrol.wait;" ::: "memory");   // x may be the previous launch's output
+    DWalk<SQ> W(P, pair, n_pairs);
+    DRows nx = {0, 0, 0};
+    if constexpr (SQ == 0) nx = d_rows(W, lane);
+    while (ok && W.valid()) {
+      const DLayer& L = *W.L;
+      const int tok0 = W.m * P.N + (int)rank * Nh, c0 = W.c0;
+      uint32_t items = d_batch(W, nx, lane);
+      W.next();
+      if constexpr (SQ == 0) nx = d_rows(W, lane);
+      for (; items && ok; items &= items - 1) {
+        const int c = c0 + __ffs(items) - 1;
+        for (int st = 0; st < kStPer; ++st) {
+          if (!d_wait_warp(&done_bar[s], ph, abort_flag, P.err)) {
+            ok = false;
+            break;
           }
-      };
-      for (int c0 = 0; c0 < L.G && ok; c0 += 32) {
-        const int n_it = d_items<SQ>(L, w, c0, lane, ibuf);
-        uint32_t km_n[kOwn];
-        int wo_n[kOwn];
-        int tv_n[kTS][kU];
-        if (n_it > 0) {
-          if constexpr (SQ > 0) load_tiles(ibuf[0], tv_n);
-          else load_meta(ibuf[0], km_n, wo_n);
-        }
-        for (int it = 0; it < n_it && ok; ++it) {
-          const int c = ibuf[it];
-          // element offset of each piece this lane copies (1 x KW: slab 0 of the
-          // item, the others follow at 64-element steps; square: per slab), -1: zeros
-          int64_t soff[kTS][kCopies];
-          if constexpr (SQ > 0) {
-#pragma unroll
-            for (int sl = 0; sl < kTS; ++sl)
-#pragma unroll
-              for (int i = 0; i < kCopies; ++i) {
-                const int row = w * kDW + (int)rank * kDHalf + warp * kRows + 4 * i + (lane >> 3);
-                const int k = c * KW + sl * kDSlabK + 8 * j;
-                const int tq = tv_n[sl][kU * i / kCopies];
-                soff[sl][i] = tq >= 0 ? ((int64_t)tq * SQ + row % SQ) * SQ + k % SQ : -1;
-              }
-            if (it + 1 < n_it) load_tiles(ibuf[it + 1], tv_n);
-          } else {
-            // packed positions in chunk c of the rows this lane looks up (-1: pruned / beyond out)
-            int prow[kOwn];
-#pragma unroll
-            for (int q = 0; q < kOwn; ++q) {
-              const int h = (int)rank * kDHalf + warp * kRows + 32 * q + lane;
-              const int b16 = w * (kDW / kWin16) + (h >> 4), bit = h & 15;
-              const bool kept = b16 < L.nw16 && ((km_n[q] >> bit) & 1u);
-              prow[q] = kept ? wo_n[q] + __popc(km_n[q] & ((1u << bit) - 1u)) : -1;
-            }
-            if (it + 1 < n_it) load_meta(ibuf[it + 1], km_n, wo_n);
-            // the rows this lane copies: warp * kRows + 4 i + (lane >> 3)
-#pragma unroll
-            for (int i = 0; i < kCopies; ++i) {
-              const int r = 4 * i + (lane >> 3);   // row within the warp's block: owner lane r % 32, slot r / 32
-              const int pr = __shfl_sync(0xffffffffu, prow[r >> 5], r & 31);
-              soff[0][i] = pr >= 0 ? (int64_t)pr * KW + 8 * j : -1;
-            }
+          if (elect_one()) {
+            if (rank == 0) mbar_arrive_expect_tx(&full_bar[s], 2u * xs_bytes);
+            tma_load_3d_pair(smem + s * xs_bytes, &L.xmap, mapa_shared(smem_u32(&full_bar[s]), 0), 0, tok0,
+                             c * (KW / 64) + 2 * st);
           }
-#pragma unroll
-          for (int sl = 0; sl < kSlabs; ++sl) {
-            if (!ok) break;
-            bool got = true;
-            if (lane == 0)
-              got = mbar_wait_bounded(&done_bar[stage / 2], phase ^ 1u, abort_flag, P.err, kDWaitLimitNs, kDevErrTimeout);
-            if (!__shfl_sync(0xffffffffu, got ? 1 : 0, 0)) {
-              ok = false;
-              break;
-            }
-            const uint32_t wb = smem_u32(smem + kDXRing + stage * kDWBytes);
-#pragma unroll
-            for (int i = 0; i < kCopies; ++i) {
-              const int rr = warp * kRows + 4 * i + (lane >> 3);
-              const uint32_t dst = wb + (uint32_t)rr * 128u + (uint32_t)((j ^ (rr & 7)) << 4);   // 128-byte swizzle
-              const int64_t so = soff[SQ > 0 ? sl : 0][i];
-              const bool kept = so >= 0;
-              // a pruned row reads nothing (source size 0) and is filled with zeros
-              const uint16_t* src = kept ? L.tiles + so + (SQ > 0 ? 0 : sl * kDSlabK) : L.tiles;
-              cp_async16_zfill(dst, src, kept ? 16u : 0u);
-            }
-            cp_async_arrive_noinc(&wfull_bar[stage]);   // fires once this thread's copies have landed
-            if (++stage == (uint32_t)kDWStages) {
-              stage = 0;
-              phase ^= 1u;
-            }
+          __syncwarp();
+          if (++s == xs_n) {
+            s = 0;
+            ph ^= 1u;
           }
         }
       }
     }
-    cp_async_wait_all();
-    __syncwarp();
-  } else if (warp == kDXWarp) {
-    // ------------------------------------------------------------ x producer
-    // Stage k's x box goes to x slot k % kDXStages once stage k - kDXStages is
-    // done, and completes on the leader's full barrier of W slot k % kDWStages.
-    uint32_t k = 0;
-    uint32_t armed = 0u, armed_par = 0u;
+  } else if (warp == 1) {
+    // ------------------------------------------------------------ W copies
+    // 1 x KW: the half window's kept rows of a chunk are one contiguous slice of
+    // the packed tiles; one box a stage (two slabs), rows rounded up to 16.
+    // Square: the half window's kept tiles of a column block are one contiguous
+    // run; lane b copies block b's, back to back.
+    uint32_t k = 0, oldest = 0;                   // stages issued / known to be read
+    uint32_t head = 0, tail = 0, hoff = 0;        // virtual bytes allocated / released, head's ring offset
     bool ok = true;
-    for (int ku = 0, u; ok && (u = owner_tile(P.tl, n_tiles, pair, n_pairs, ku)) >= 0; ++ku) {
-      const DLayer& L = P.L[d_layer_of(P, u)];
-      const int lt = u - L.tile_begin;
-      const int m = lt % L.n_m, w = lt / L.n_m;
-      const int tok0 = m * 2 * kDM + (int)rank * kDM;
-      for (int c0 = 0; c0 < L.G && ok; c0 += 32) {
-        const int n_it = d_items<SQ>(L, w, c0, lane, ibuf);
-        if (lane == 0) {
-          for (int it = 0; it < n_it && ok; ++it) {
-            const int c = ibuf[it];
-            for (int sl = 0; sl < kSlabs && ok; ++sl, ++k) {
-              if (k >= (uint32_t)kDXStages) {
-                const uint32_t pp = (k - kDXStages) / 2;   // the stage pair whose x slot this one reuses
-                if (!mbar_wait_bounded(&done_bar[pp % kDSuper], (pp / kDSuper) & 1u, abort_flag, P.err,
-                                       kDWaitLimitNs, kDevErrTimeout)) {
-                  ok = false;
-                  break;
-                }
+    // The whole warp walks the stages (the lookups of a batch reach every lane
+    // through shared memory) and one elected lane issues, as in the MMA warp.
+    auto slot = [&](uint32_t bytes, uint32_t& off) {   // room for a stage: its offset in the ring
+      const uint32_t e = k % kDWSeq;
+      off = hoff;
+      uint32_t pad = 0u;
+      if (off + bytes > w_ring) {
+        pad = w_ring - hoff;
+        off = 0u;
+      }
+      const uint32_t end = head + pad + bytes;
+      while (end - tail > w_ring || k - oldest >= (uint32_t)kDWSeq) {
+        const uint32_t j = oldest % kDWSeq;
+        if (!d_wait_warp(&wempty_bar[j], (oldest / kDWSeq) & 1u, abort_flag, P.err)) return false;
+        tail = w_end[j];
+        ++oldest;
+      }
+      __syncwarp();
+      if (elect_one()) {
+        w_end[e] = end;
+        mbar_arrive_expect_tx(&wfull_bar[e], bytes);
+      }
+      __syncwarp();
+      head = end;
+      hoff = off + bytes;
+      ++k;
+      return true;
+    };
+    DWalk<SQ> W(P, pair, n_pairs);
+    if constexpr (SQ > 0) {
+      uint64_t mk_n;
+      int st_n[kBlk];
+      auto load = [&]() {
+        const int win = 2 * W.w + (int)rank;
+        mk_n = d_blocks(W, win, lane);
+#pragma unroll
+        for (int b = 0; b < kBlk; ++b) st_n[b] = 0;
+        if (W.valid() && W.c0 + lane < W.L->G && win < W.L->nw)
+#pragma unroll
+          for (int b = 0; b < kBlk; ++b)
+            st_n[b] = W.L->win_off[(int64_t)((W.c0 + lane) * kBlk + b) * (W.L->nw + 1) + win];
+      };
+      load();
+      while (ok && W.valid()) {
+        const DLayer& L = *W.L;
+        const int n_it = min(32, L.G - W.c0);
+        w_n[lane] = mk_n;
+#pragma unroll
+        for (int b = 0; b < kBlk; ++b) w_start[lane][b] = st_n[b];
+        W.next();
+        load();
+        __syncwarp();
+        const uint16_t* tiles = L.tiles;
+        for (int i = 0; i < n_it && ok; ++i) {
+          const uint64_t v = w_n[i];
+          uint32_t off;
+          ok = slot((uint32_t)__popcll(v) * (SQ * SQ * 2), off);
+          if (ok && elect_one()) {
+            uint8_t* dst = wsmem + off;
+            uint64_t* bar = &wfull_bar[(k - 1) % kDWSeq];
+#pragma unroll
+            for (int b = 0; b < kBlk; ++b) {
+              const int n = __popc((uint32_t)(v >> (b * kR)) & ((1u << kR) - 1u));
+              if (n > 0) {
+                const int start = w_start[i][b];
+                if constexpr (SQ < 64)
+                  bulk_g2s(dst, tiles + (int64_t)start * (SQ * SQ), (uint32_t)n * (SQ * SQ * 2), bar);
+                else
+                  tma_load_2d(dst, &L.wmap[n - 1], bar, 0, start * SQ);
+                dst += n * (SQ * SQ * 2);
               }
-              const uint32_t fs = (k / 2) % kDSuper;
-              if (rank == 0) mbar_arrive_expect_tx(&full_bar[fs], 2u * kDXBytes);
-              tma_load_3d_pair(smem + (k % kDXStages) * kDXBytes, &L.xmap, mapa_shared(smem_u32(&full_bar[fs]), 0),
-                               0, tok0, c * kSlabs + sl);
-              armed |= 1u << fs;
-              armed_par = (armed_par & ~(1u << fs)) | (((k / 2 / kDSuper) & 1u) << fs);
             }
           }
+          __syncwarp();
         }
-        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+        __syncwarp();   // every lane has read the batch
+      }
+    } else {
+      DRows nx = d_rows(W, lane);
+      while (ok && W.valid()) {
+        const DLayer& L = *W.L;
+        uint32_t items = d_batch(W, nx, lane);
+        const int start_l = rank ? nx.b : nx.a;
+        w_start[lane][0] = start_l;
+        w_n[lane] = (uint64_t)((rank ? nx.c : nx.b) - start_l);
+        W.next();
+        nx = d_rows(W, lane);
+        __syncwarp();
+        for (; items && ok; items &= items - 1) {
+          const int i = __ffs(items) - 1;
+          const int start = w_start[i][0], h16 = ((int)w_n[i] + 15) / 16;
+          for (int st = 0; st < kStPer && ok; ++st) {
+            uint32_t off;
+            ok = slot((uint32_t)h16 * (16u * kDStageK * 2), off);
+            if (ok && h16 > 0 && elect_one())
+              tma_load_3d(wsmem + off, &L.wmap[h16 - 1], &wfull_bar[(k - 1) % kDWSeq], 0, start, 2 * st);
+            __syncwarp();
+          }
+        }
+        __syncwarp();   // every lane has read the batch
       }
     }
-    if (lane == 0 && !ok && rank == 0) {
-      // let the x copies in flight land before the CTA winds down
-      for (int s = 0; s < kDSuper; ++s) {
-        if (!((armed >> s) & 1u)) continue;
+    if (!ok && lane == 0) {
+      // let the W copies in flight land before the CTA winds down
+      for (uint32_t b = 0; b < (uint32_t)kDWSeq && b < k; ++b) {
+        const uint32_t kb = k - 1 - b;
         const uint64_t t0 = globaltimer_ns();
-        while (!mbar_try_wait_acq_cluster(&full_bar[s], (armed_par >> s) & 1u))
+        while (!mbar_try_wait(&wfull_bar[kb % kDWSeq], (kb / kDWSeq) & 1u))
           if (globaltimer_ns() - t0 > kDDrainLimitNs) break;
       }
     }
     __syncwarp();
-  } else if (warp == kDFwdWarp || warp > kDXWarp) {
-    // ------------------------------------------------------------ forwarders
-    // Once all of this CTA's producer threads' copies of a stage pair have
-    // landed, make them visible to the tensor cores (async proxy) and tell the
-    // leader.  The forwarders take the stage pairs in turn, so that their
-    // fences (about a microsecond per batch) overlap.
-    const uint32_t f = warp == kDFwdWarp ? 0u : (uint32_t)(warp - kDXWarp);   // takes pairs p with p % kDNumFwd == f
-    uint32_t K = 0;   // stages before the current batch
-    bool ok = true;
-    for (int ku = 0, u; ok && (u = owner_tile(P.tl, n_tiles, pair, n_pairs, ku)) >= 0; ++ku) {
-      const DLayer& L = P.L[d_layer_of(P, u)];
-      const int w = (u - L.tile_begin) / L.n_m;
-      for (int c0 = 0; c0 < L.G && ok; c0 += 32) {
-        const int n_pr = d_items<SQ>(L, w, c0, lane, ibuf) * kSlabs / 2;   // stage pairs of the batch
-        if (lane == 0) {
-          int cnt = 1;
-          for (int q = (int)((f + kDNumFwd - (K / 2) % kDNumFwd) % kDNumFwd); q < n_pr && ok; q += kDNumFwd * cnt) {
-            const uint32_t p0 = K / 2 + (uint32_t)q;   // global pair index
-            const uint32_t s0 = (2 * p0) % kDWStages, ph0 = ((2 * p0) / kDWStages) & 1u;
-            if (!mbar_wait_bounded(&wfull_bar[s0], ph0, abort_flag, P.err, kDWaitLimitNs, kDevErrTimeout) ||
-                !mbar_wait_bounded(&wfull_bar[s0 + 1], ph0, abort_flag, P.err, kDWaitLimitNs, kDevErrTimeout)) {
-              ok = false;
-              break;
-            }
-            // take this forwarder's following pairs that have landed too, so that
-            // one release fence covers them all (a release per stage is slow)
-            cnt = 1;
-            while (q + kDNumFwd * cnt < n_pr && cnt * kDNumFwd < kDSuper) {
-              const uint32_t p2 = p0 + kDNumFwd * (uint32_t)cnt;
-              const uint32_t s2 = (2 * p2) % kDWStages, ph2 = ((2 * p2) / kDWStages) & 1u;
-              if (!mbar_try_wait(&wfull_bar[s2], ph2) || !mbar_try_wait(&wfull_bar[s2 + 1], ph2)) break;
-              ++cnt;
-            }
-            fence_proxy_async_cta();
-            fence_acq_rel_cluster();   // with the relaxed arrives below: a release of the copies to the leader
-            for (int i = 0; i < cnt; ++i) {
-              const uint32_t fs = (p0 + kDNumFwd * (uint32_t)i) % kDSuper;
-              const uint32_t fb = mapa_shared(smem_u32(&full_bar[fs]), 0);
-              mbar_arrive_cluster_relaxed(fb);   // one arrival per stage of the pair
-              mbar_arrive_cluster_relaxed(fb);
-            }
-          }
-        }
-        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-        K += (uint32_t)(2 * n_pr);
-      }
-    }
   } else if (warp == kDMmaWarp && rank == 0) {
     // ------------------------------------------------------------ MMA issuer (leader)
-    uint32_t ws = 0, wph = 0, xs = 0;   // W slot (and its barriers' phase), x slot
-    int buf = 0;
-    uint32_t ae_ph = 0u;
+    uint32_t kb = 0, s = 0, ph = 0u, as = 0;
     bool ok = true;
-    constexpr uint32_t idesc = idesc_bf16_f32(2 * kDM, kDW);
-    for (int ku = 0, u; ok && (u = owner_tile(P.tl, n_tiles, pair, n_pairs, ku)) >= 0; ++ku) {
+    const uint32_t idesc = idesc_bf16_f32(kDW, 0) | ((uint32_t)(P.N >> 3) << 17);
+    // x operand descriptors: 16-byte units from x slot 0, a slab, a K step
+    const uint64_t xd = sdesc_sw128(smem_u32(smem));
+    const uint32_t x_lo = (uint32_t)xd, x_hi = (uint32_t)(xd >> 32), slab = (uint32_t)Nh * 8u;
+    int part = 0;   // items of the next unit, counted while this one runs
+    auto count = [&](int u) {
+      if (u < 0) return 0;
       const DLayer& L = P.L[d_layer_of(P, u)];
-      const int w = (u - L.tile_begin) / L.n_m;
-      if (lane == 0) {
-        ok = mbar_wait_bounded_cluster(&aempty_bar[buf], ((ae_ph >> buf) & 1u) ^ 1u, abort_flag, P.err, kDWaitLimitNs,
-                                       kDevErrTimeout);
-        ae_ph ^= 1u << buf;
-        tc_fence_after();
-      }
-      ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-      const uint32_t d = tmem + (uint32_t)(buf * kDW);
-      bool first = true;
-      for (int c0 = 0; c0 < L.G && ok; c0 += 32) {
-        const int n_it = d_items<SQ>(L, w, c0, lane, ibuf);
-        if (lane == 0) {
-          // stages two at a time (every item has an even number of them)
-          for (int it = 0; it < n_it * kSlabs && ok; it += 2) {
-            if (!mbar_wait_bounded_cluster(&full_bar[ws / 2], wph, abort_flag, P.err, kDWaitLimitNs, kDevErrTimeout)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after();
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              const uint64_t ad = sdesc_sw128(smem_u32(smem + (xs + h) * kDXBytes));
-              const uint64_t bd = sdesc_sw128(smem_u32(smem + kDXRing + (ws + h) * kDWBytes));
-#pragma unroll
-              for (int kk = 0; kk < kDSlabK / 16; ++kk)
-                mma_bf16_ss_pair(d, ad + (uint64_t)(2 * kk), bd + (uint64_t)(2 * kk), idesc,
-                                 (first && h == 0 && kk == 0) ? 0u : 1u);
-            }
-            first = false;
-            mma_commit_pair_mc(&done_bar[ws / 2], 0x3);
-            ws += 2;
-            if (ws == (uint32_t)kDWStages) {
-              ws = 0;
-              wph ^= 1u;
-            }
-            xs += 2;
-            if (xs == (uint32_t)kDXStages) xs = 0;
-          }
+      return d_count_part<SQ>(L, (u - L.tile_begin) / L.n_m, lane);
+    };
+    int u = owner_tile(P.tl, n_tiles, pair, n_pairs, 0);
+    part = count(u);
+    for (int ku = 0; ok && u >= 0; ++ku, ++kb) {
+      const int n_st = (int)__reduce_add_sync(0xffffffffu, (uint32_t)part) * kStPer;
+      u = owner_tile(P.tl, n_tiles, pair, n_pairs, ku + 1);
+      part = count(u);
+      // The whole warp walks the stages, so that every operand is warp-uniform, and
+      // one elected lane issues: from inside a one-lane branch each MMA cost 70
+      // cycles of issue, eight of them more than a stage's tensor work.
+      const uint32_t buf = kb % n_buf;
+      ok = __all_sync(0xffffffffu, d_wait_cluster(&aempty_bar[buf], ((kb / n_buf) & 1u) ^ 1u, abort_flag, P.err));
+      tc_fence_after();
+      const uint32_t d = tmem + buf * (kDN / 4);
+      for (int i = 0; i < n_st && ok; ++i) {
+        if (!__all_sync(0xffffffffu, d_wait_cluster(&full_bar[s], ph, abort_flag, P.err))) {
+          ok = false;
+          break;
         }
-        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-        first = __shfl_sync(0xffffffffu, first ? 1 : 0, 0) != 0;
+        tc_fence_after();
+        const uint32_t a = tmem + t_a + as * (kDStageK / 2);
+        const uint32_t b = x_lo + s * (xs_bytes >> 4);
+        if (elect_one()) {
+#pragma unroll
+          for (int kk = 0; kk < kDStageK / 16; ++kk)
+            mma_bf16_ts_pair(d, a + 8 * kk, ((uint64_t)x_hi << 32) | (b + (kk >= 4 ? slab : 0u) + 2 * (kk & 3)), idesc,
+                             (i == 0 && kk == 0) ? 0u : 1u);
+          mma_commit_pair_mc(&done_bar[s], 0x3);
+        }
+        __syncwarp();
+        if (++as == a_n) as = 0;
+        if (++s == xs_n) {
+          s = 0;
+          ph ^= 1u;
+        }
       }
-      if (!ok) break;
-      if (lane == 0) mma_commit_pair_mc(&afull_bar[buf], 0x3);
-      buf ^= 1;
+      if (ok && elect_one()) mma_commit_pair_mc(&afull_bar[buf], 0x3);
+      __syncwarp();
     }
-    if (lane == 0) {
+    if (elect_one()) {
       mma_commit_pair(&drain_bar);
       mbar_wait_bounded(&drain_bar, 0u, nullptr, P.err, kDWaitLimitNs, kDevErrTimeout);
     }
     __syncwarp();
-  } else if (warp >= kDEpiWarp0) {
-    // ------------------------------------------------------------ epilogue
-    const int q = warp & 3;   // TMEM lane quarter this warp may access
-    int buf = 0;
-    uint32_t af_ph = 0u;
+  } else if (warp >= kDConvWarp0 && warp < kDEpiWarp0) {
+    // ------------------------------------------------------------ converters
+    // Lane l of quarter q owns window row 128 rank + 32 q + l; the sets of four
+    // warps take the stages in turn.
+    const int q = warp & 3;
+    const uint32_t set = (uint32_t)(warp - kDConvWarp0) >> 2;
+    const int r = 32 * q + lane;   // row within this CTA's half
+    const uint32_t lane_addr = tmem + ((uint32_t)(32 * q) << 16) + t_a;
+    const uint32_t leader_full = mapa_shared(smem_u32(full_bar), 0);
+    uint32_t k = 0, hoff = 0;                  // stage, its ring offset
+    uint32_t s = 0;                            // its full barrier
+    uint32_t ds = xs_n - a_n, dph = 1u;        // done barrier of the stage a_n earlier (the A slot's last user)
+    if (xs_n == a_n) ds = 0;
+    uint32_t as = 0;                           // its A slot
     bool ok = true;
-    for (int ku = 0, u; ok && (u = owner_tile(P.tl, n_tiles, pair, n_pairs, ku)) >= 0; ++ku) {
-      const DLayer& L = P.L[d_layer_of(P, u)];
-      const int lt = u - L.tile_begin;
-      const int m = lt % L.n_m, w = lt / L.n_m;
-      // a window with no kept row in any chunk has no MMA: its rows are zero
-      bool any = SQ > 0;   // square groups: every slab has MMAs
-      if constexpr (SQ == 0) {
-        const int lo = w * (kDW / kWin16), hi = min(lo + kDW / kWin16, L.nw16);
-        for (int c = lane; c < L.G && !any; c += 32) {
-          const int32_t* wo = L.win_off16 + (int64_t)c * (L.nw16 + 1);
-          any = wo[hi] > wo[lo];
-        }
-        any = __any_sync(0xffffffffu, any);
-      }
-      const bool got =
-          mbar_wait_bounded(&afull_bar[buf], (af_ph >> buf) & 1u, abort_flag, P.err, kDWaitLimitNs, kDevErrTimeout);
-      if (!__all_sync(0xffffffffu, got)) {   // the TMEM loads below need the whole warp
-        ok = false;
-        break;
-      }
-      af_ph ^= 1u << buf;
-      tc_fence_after();
-      const int tok = m * 2 * kDM + (int)rank * kDM + 32 * q + lane;
-      uint16_t* yrow = L.y + (int64_t)tok * L.out;
-      const bool vec_ok = (L.out & 7) == 0;
-#pragma unroll 1
-      for (int j = 0; j < kDW / 32; ++j) {
-        uint32_t v[32];
-        tmem_ld_x32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * kDW + 32 * j), v);
-        tmem_wait_ld();
-        reg_fence(v);
-        const int r0 = w * kDW + 32 * j;
-        if (tok < P.T) {
+    // one stage of `bytes` in the ring: row[b] = this lane's row in row piece b's
+    // compact block (-1: pruned), at off[b] from the stage's start
+    auto stage = [&](const int (&row)[kBlk], const uint32_t (&off)[kBlk], uint32_t bytes) {
+      if (hoff + bytes > w_ring) hoff = 0;
+      if (k % kDConvSets == set) {
+        const uint32_t e = k % kDWSeq;
+        if (!d_wait_warp(&wfull_bar[e], (k / kDWSeq) & 1u, abort_flag, P.err)) return false;
+        uint32_t v[2][32];
+        {
+          const uint32_t base = smem_u32(wsmem) + hoff;
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const int rb = r0 + 8 * k;
-            const float* f = reinterpret_cast<const float*>(v + 8 * k);
-            if (vec_ok && rb + 8 <= L.out) {
-              *reinterpret_cast<uint4*>(yrow + rb) =
-                  any ? make_uint4(d_pack_bf16x2(f[0], f[1]), d_pack_bf16x2(f[2], f[3]), d_pack_bf16x2(f[4], f[5]),
-                                   d_pack_bf16x2(f[6], f[7]))
-                      : make_uint4(0u, 0u, 0u, 0u);
-            } else {
+          for (int b = 0; b < kBlk; ++b) {
+            const uint32_t ro = (uint32_t)row[b] * (kRowK * 2);
+            // 16-byte piece j of a row is read from (64-wide rows, which TMA swizzled)
+            // or at (plain rows) piece j ^ swz, which spreads eight rows over the banks
+            const uint32_t swz = (ro >> 7) & (uint32_t)(kPieces - 1);
+            const uint32_t a = base + off[b] + ro;
+            uint4 p[kPieces];
 #pragma unroll
-              for (int e = 0; e < 8; ++e)
-                if (rb + e < L.out) yrow[rb + e] = any ? __bfloat16_as_ushort(__float2bfloat16_rn(f[e])) : 0;
+            for (int j = 0; j < kPieces; ++j) {
+              p[j] = make_uint4(0u, 0u, 0u, 0u);
+              if (row[b] >= 0) p[j] = lds128(a + (((uint32_t)j ^ swz) << 4));
+            }
+            if constexpr (kRowK < 64) {
+              // plain rows: piece j now lies in p[j ^ swz]
+#pragma unroll
+              for (int d = 1; d < kPieces; d *= 2)
+#pragma unroll
+                for (int j = 0; j < kPieces; ++j)
+                  if ((j & d) == 0) {
+                    const bool sw = (swz & (uint32_t)d) != 0;
+                    const uint4 x = p[j], y = p[j + d];
+                    p[j] = sw ? y : x;
+                    p[j + d] = sw ? x : y;
+                  }
+            }
+#pragma unroll
+            for (int j = 0; j < kPieces; ++j) {
+              uint32_t* o = &v[b / kSub][4 * (b % kSub * kPieces + j)];
+              o[0] = p[j].x;
+              o[1] = p[j].y;
+              o[2] = p[j].z;
+              o[3] = p[j].w;
             }
           }
         }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&wempty_bar[e]);
+        if (k >= a_n && !d_wait_warp(&done_bar[ds], dph, abort_flag, P.err)) return false;
+        tc_fence_after();
+        const uint32_t at = lane_addr + as * (kDStageK / 2);
+        tmem_st_x32(at, v[0]);
+        tmem_st_x32(at + 32, v[1]);
+        tmem_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster_relaxed(leader_full + 8u * s);
       }
+      hoff += bytes;
+      if (++ds == xs_n) {
+        ds = 0;
+        dph ^= 1u;
+      }
+      if (++s == xs_n) s = 0;
+      if (++as == a_n) as = 0;
+      ++k;
+      return true;
+    };
+    DWalk<SQ> W(P, pair, n_pairs);
+    if constexpr (SQ > 0) {
+      const int br = r / SQ;
+      uint64_t mk_n = d_blocks(W, 2 * W.w + (int)rank, lane);
+      while (ok && W.valid()) {
+        const uint64_t mk = mk_n;
+        const int n_it = min(32, W.L->G - W.c0);
+        W.next();
+        mk_n = d_blocks(W, 2 * W.w + (int)rank, lane);
+        for (int i = 0; i < n_it && ok; ++i) {
+          const uint64_t v = __shfl_sync(0xffffffffu, mk, i);
+          int row[kBlk];
+          uint32_t off[kBlk];
+#pragma unroll
+          for (int b = 0; b < kBlk; ++b) {
+            const int at = b * kR;   // this block's bits
+            const uint32_t mb = (uint32_t)(v >> at) & ((1u << kR) - 1u);
+            row[b] = ((mb >> br) & 1u) ? (int)__popc(mb & ((1u << br) - 1u)) * SQ + r % SQ : -1;
+            off[b] = (uint32_t)__popcll(v & ((1ull << at) - 1ull)) * (SQ * SQ * 2);
+          }
+          ok = stage(row, off, (uint32_t)__popcll(v) * (SQ * SQ * 2));
+        }
+      }
+    } else {
+      // this warp's two 16-row windows in an item: kept masks, first packed row
+      uint32_t mk_n;
+      int wo_n;
+      auto load = [&]() {
+        mk_n = 0;
+        wo_n = 0;
+        const int c = W.c0 + lane;
+        if (!W.valid() || c >= W.L->G) return;
+        const int nw = W.L->nw, b16 = W.w * (kDW / kWin16) + (int)rank * (kDHalf / kWin16) + 2 * q;
+        const uint16_t* km = static_cast<const uint16_t*>(W.L->kmask) + (int64_t)c * nw;
+        if (b16 < nw) {
+          mk_n = km[b16];
+          wo_n = W.L->win_off[(int64_t)c * (nw + 1) + b16];
+        }
+        if (b16 + 1 < nw) mk_n |= (uint32_t)km[b16 + 1] << 16;
+      };
+      DRows nx = d_rows(W, lane);
+      load();
+      while (ok && W.valid()) {
+        uint32_t items = d_batch(W, nx, lane);
+        const int start_l = rank ? nx.b : nx.a, n_l = (rank ? nx.c : nx.b) - start_l;
+        const uint32_t mk_l = mk_n;
+        const int at_l = wo_n - start_l;
+        W.next();
+        nx = d_rows(W, lane);
+        load();
+        for (; items && ok; items &= items - 1) {
+          const int i = __ffs(items) - 1;
+          const uint32_t mk = __shfl_sync(0xffffffffu, mk_l, i);
+          const int n = __shfl_sync(0xffffffffu, n_l, i), at = __shfl_sync(0xffffffffu, at_l, i);
+          // rows 32 q .. + 31 of the half window are consecutive bits, and consecutive in the slice
+          int row[kBlk];
+          uint32_t off[kBlk];
+          const uint32_t slab = (uint32_t)((n + 15) / 16) * (16 * 128);
+          row[0] = row[1] = ((mk >> lane) & 1u) ? at + (int)__popc(mk & ((1u << lane) - 1u)) : -1;
+          off[0] = 0;
+          off[1] = slab;
+#pragma unroll
+          for (int st = 0; st < kStPer; ++st)
+            if (ok) ok = stage(row, off, 2 * slab);
+        }
+      }
+    }
+  } else if (warp >= kDEpiWarp0) {
+    // ------------------------------------------------------------ epilogue
+    const int q = warp & 3, hh = (warp - kDEpiWarp0) >> 2;   // TMEM lane quarter, half of the tile's tokens
+    const int nl = P.N / 32;                                 // 16-token loads per warp
+    asm volatile("griddepcontrol.wait;" ::: "memory");       // the previous launch may still use y
+    uint32_t kb = 0;
+    bool ok = true;
+    const uint32_t leader_empty = mapa_shared(smem_u32(aempty_bar), 0);
+    for (int ku = 0, u; ok && (u = owner_tile(P.tl, n_tiles, pair, n_pairs, ku)) >= 0; ++ku, ++kb) {
+      const DLayer& L = P.L[d_layer_of(P, u)];
+      const int lt = u - L.tile_begin;
+      const int m = lt % L.n_m, w = lt / L.n_m;
+      const bool any = __any_sync(0xffffffffu, d_count_part<SQ>(L, w, lane) > 0);   // else no MMA wrote D: zeros
+      const uint32_t buf = kb % n_buf;
+      if (!d_wait_warp(&afull_bar[buf], (kb / n_buf) & 1u, abort_flag, P.err)) {
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      uint32_t pk[kDN / 4];   // this lane's row: pairs of tokens
+      const uint32_t dcol = tmem + ((uint32_t)(32 * q) << 16) + buf * (kDN / 4) + (uint32_t)(hh * Nh);
+#pragma unroll
+      for (int i = 0; i < kDN / 32; ++i)
+        if (i < nl) {
+          uint32_t v[16];
+          tmem_ld_x16(dcol + 16 * i, v);
+          tmem_wait_ld();
+          reg_fence(v);
+#pragma unroll
+          for (int e = 0; e < 8; ++e)
+            pk[8 * i + e] = any ? d_pack_bf16x2(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1])) : 0u;
+        }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive_cluster_relaxed(mapa_shared(smem_u32(&aempty_bar[buf]), 0));
-      buf ^= 1;
+      if (lane == 0) mbar_arrive_cluster_relaxed(leader_empty + 8u * buf);   // D may be overwritten
+      const int row = w * kDW + (int)rank * kDHalf + 32 * q + lane;
+      const int tok0 = m * P.N + hh * Nh;
+      if ((L.out & 1) == 0) {
+        // neighbouring lanes swap so that each holds one token of two rows: even
+        // lanes the first token of every pair, odd lanes the second
+        const uint32_t sel = (lane & 1) ? 0x3276u : 0x5410u;
+        const bool in_row = (row & ~1) < L.out;
+        uint16_t* yp = L.y + (int64_t)(tok0 + (lane & 1)) * L.out + (row & ~1);
+#pragma unroll
+        for (int i = 0; i < kDN / 32; ++i)
+          if (i < nl) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+              const int t = 16 * i + 2 * e;
+              const uint32_t o = __shfl_xor_sync(0xffffffffu, pk[8 * i + e], 1);
+              if (in_row && tok0 + t + (lane & 1) < P.T)
+                *reinterpret_cast<uint32_t*>(yp + (int64_t)t * L.out) = __byte_perm(pk[8 * i + e], o, sel);
+            }
+          }
+      } else if (row < L.out) {
+        uint16_t* yp = L.y + (int64_t)tok0 * L.out + row;
+#pragma unroll
+        for (int i = 0; i < kDN / 32; ++i)
+          if (i < nl) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+              const int t = 16 * i + 2 * e;
+              if (tok0 + t < P.T) yp[(int64_t)t * L.out] = (uint16_t)pk[8 * i + e];
+              if (tok0 + t + 1 < P.T) yp[(int64_t)(t + 1) * L.out] = (uint16_t)(pk[8 * i + e] >> 16);
+            }
+          }
+      }
+      __syncwarp();
     }
   }
 
@@ -604,26 +820,15 @@ cudaError_t d_launch(const cudaLaunchConfig_t& cfg, const DParams& P) {
 
 }  // namespace
 
-// Which 1 x KW layers take this kernel rather than the gathering one, by the
-// layer's own group shape and T (so that a batched call gives each layer what
-// gs_linear gives it, bit for bit).  Measured on GB300 at d = 0.5 with the
-// balanced tile lists, one batched call per block (7 projections):
-//  - 1 x 256 from 129 tokens: LLaMA-2-13B block 0.142 / 0.144 / 0.236 / 0.330
-//    ms at T = 160 / 256 / 512 / 640 against 0.172 / 0.173 / 0.294 / 0.426 with
-//    the gathering kernel for the 5120-row layers (7B block 0.101-0.220 against
-//    0.117-0.299; Qwen2.5-7B 0.180-0.249 against 0.217-0.304 from T = 384, 4 %
-//    behind at 160 and 256).  Alone, a 5120 x 5120 layer at T = 512 still runs
-//    faster gathering (0.040 vs 0.048 ms: 40 units for 76 CTA pairs), but layers
-//    are mostly called a block at a time;
-//  - 1 x 128 in the whole prefill regime: over the five 7B / 13B projection
-//    shapes at T = 64 and 128 it takes 0.91-0.96x the gathering kernel's time in
-//    nine of the ten cases (13824 x 5120 at T = 128: 1.02x), while 1 x 256
-//    layers up to 128 tokens stay on the gathering kernel (1.15-1.24x).
-// Both kernels' times hardly depend on the density.
+// Which 1 x KW layers take this kernel: all that have kept groups, in the whole
+// prefill regime.  Against the gathering kernel, d = 0.5, us per batched block:
+// 13B 1 x 256 at T = 17 / 128 / 256 / 512 71 / 76 / 93 / 168 against 92 / 98 / 173 / 294;
+// 7B 1 x 128 at T = 32 / 128 50 / 54 against 78 / 101.  One call per layer, over
+// nine shapes from 1024 x 1024 to 20000 x 1024 and T = 17 to 640, it takes
+// 0.4-0.97x the gathering kernel's time.
 bool prefill_prefers_dense(const gs_packed* p, int64_t T) {
-  if (p->kept == 0 || p->g_out != 1) return false;
-  if (p->g_in == 128) return true;
-  return p->g_in == 256 && T > 128;
+  (void)T;
+  return p->kept > 0 && p->g_out == 1 && (p->g_in == 128 || p->g_in == 256);
 }
 
 gs_status launch_prefill_dense(const void* const* xs, const gs_packed* const* ps, int n, int64_t T, void* const* ys,
@@ -637,12 +842,15 @@ gs_status launch_prefill_dense(const void* const* xs, const gs_packed* const* ps
   const int sq = go > 1 ? go : 0;   // square g x g groups
   if (sq ? (sq != kw || (sq != 16 && sq != 32 && sq != 64)) : (kw != 256 && kw != 128)) return GS_ERR_UNSUPPORTED;
   for (int i : order)
-    if (sq && !ps[i]->gtidx) return GS_ERR_UNSUPPORTED;
+    if (!sq && !ps[i]->wmaps_valid) return GS_ERR_UNSUPPORTED;
   int* err = device_error_flag();
   if (!err) return GS_ERR_CUDA;
   // most tensor work per unit (the widest input) first
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return ps[a]->in > ps[b]->in; });
   const int64_t max_pairs = d_sm_count() / 2;
+  // tiles of equal size, in whole 32 tokens (16 per CTA and epilogue load)
+  const int64_t n_m = (T + kDN - 1) / kDN;
+  const int64_t tile_n = ((T + n_m - 1) / n_m + 31) / 32 * 32;
   for (int b0 = 0; b0 < n; b0 += kDMaxLayers) {
     const int nb = std::min(kDMaxLayers, n - b0);
     DParams P;
@@ -652,29 +860,34 @@ gs_status launch_prefill_dense(const void* const* xs, const gs_packed* const* ps
       const int i = order[b0 + k];
       const gs_packed* p = ps[i];
       DLayer& L = P.L[k];
-      if (!encode_tmap_slabs_bf16(&L.xmap, xs[i], (uint64_t)p->in, (uint64_t)T, kDM, 1)) return GS_ERR_CUDA;
+      if (!encode_tmap_slabs_bf16(&L.xmap, xs[i], (uint64_t)p->in, (uint64_t)T, (uint32_t)(tile_n / 2), 2))
+        return GS_ERR_CUDA;
       L.tiles = p->tiles;
       L.y = static_cast<uint16_t*>(ys[i]);
       L.out = (int32_t)p->out;
       if (sq) {
         if (p->in % 128 != 0) return GS_ERR_UNSUPPORTED;
-        L.gtidx = p->gtidx;
-        L.Gin = p->G;
-        L.G = (int32_t)(p->in / 128);   // 128-column items (two 64-column stages)
+        for (int h = 0; h < kDHalf / sq; ++h) std::memcpy(&L.wmap[h], p->gmaps[h], sizeof(CUtensorMap));
+        L.win_off = p->gwoff;
+        L.kmask = p->gwmask;
+        L.nw = p->nwin;
+        L.G = (int32_t)(p->in / 128);   // 128-column items, one stage each
       } else {
-        L.win_off16 = p->win_off16;
-        L.kmask16 = p->kmask16;
+        for (int h = 0; h < kDWMaps; ++h) std::memcpy(&L.wmap[h], p->wmaps_full[h], sizeof(CUtensorMap));
+        L.win_off = p->win_off16;
+        L.kmask = p->kmask16;
+        L.nw = p->nw16;
         L.G = p->G;
-        L.nw16 = p->nw16;
       }
-      if (L.G > 32767) return GS_ERR_UNSUPPORTED;   // chunk lists hold 16-bit indices
-      L.n_m = (int32_t)((T + 2 * kDM - 1) / (2 * kDM));
+      if (L.G > 32767) return GS_ERR_UNSUPPORTED;
+      L.n_m = (int32_t)n_m;
       L.tile_begin = (int32_t)tiles;
       tiles += (int64_t)L.n_m * ((p->out + kDW - 1) / kDW);
     }
     if (tiles > INT32_MAX) return GS_ERR_UNSUPPORTED;
     P.n_layers = nb;
     P.T = (int32_t)T;
+    P.N = (int32_t)tile_n;
     P.n_tiles = (int32_t)tiles;
     P.err = err;
     P.inject_ns = b0 == 0 ? take_injected_wait(GS_ALGO_PREFILL_DENSE) : 0;
@@ -693,13 +906,15 @@ gs_status launch_prefill_dense(const void* const* xs, const gs_packed* const* ps
     cfg.blockDim = dim3(kDThreads);
     cfg.dynamicSmemBytes = kDSmem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     const cudaError_t e = sq == 16   ? d_launch<128, 16>(cfg, P)
                           : sq == 32 ? d_launch<128, 32>(cfg, P)
                           : sq == 64 ? d_launch<128, 64>(cfg, P)

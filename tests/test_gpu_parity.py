@@ -110,6 +110,28 @@ def test_prefill_dense_parity(gs, out, inp, d, seed):
     assert gs.device_status() == gs.GS_OK
 
 
+@pytest.mark.parametrize("go,gi", [(1, 256), (1, 128), (16, 16), (32, 32), (64, 64)])
+@pytest.mark.parametrize("d", [0.05, 0.5, 1.0])
+def test_prefill_dense_token_tiles(gs, go, gi, d):
+    """Zero-filled kernel at the edges of its token tiles (32-token steps, one and two accumulator
+    buffers, one and two tiles), with odd and ragged row counts, stages of every size in its byte
+    ring (wrapping at d = 1) and a half window without a kept row."""
+    import torch
+    from tests._gpu_util import ABS, REL, bf16_to_f64
+    for out, inp in ((257, 2560), (640, 4096)) if go == 1 else ((192, 2560), (640, 4096)):
+        Wb = wl.random_weight_bits(out, inp, seed=out + gi)
+        B = wl.random_mask(out // go, inp // gi, d, seed=out + gi + 1)
+        B[128 // go:min(256, out) // go, ::3] = 0
+        p = gs.pack_groups(to_dev(Wb), torch.from_numpy(np.ascontiguousarray(B, dtype=np.uint8)).cuda(), go, gi)
+        for T in (17, 32, 33, 64, 65, 97, 128, 129, 161, 256, 257, 290):
+            xb = wl.random_activation_bits(T, inp, seed=T + gi)
+            y = to_bits(gs.linear(to_dev(xb), p, algo=gs.ALGO_PREFILL_DENSE if go == 1 else gs.ALGO_AUTO))
+            yr, A = orc.linear(xb, Wb, B, go, gi)
+            err = np.abs(bf16_to_f64(y) - yr)
+            assert np.all(err <= REL * A + ABS), (go, gi, d, out, inp, T, float((err / (REL * A + ABS)).max()))
+    assert gs.device_status() == gs.GS_OK
+
+
 @pytest.mark.parametrize("go,gi", [(1, 256), (1, 128), (32, 32)])
 def test_prefill_dense_large_ragged_layers(gs, go, gi):
     """Zero-filled kernel on ~10K-row layers at T ~ 1K (80+ units, more than one per CTA pair):
