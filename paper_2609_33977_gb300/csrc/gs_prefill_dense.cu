@@ -51,8 +51,7 @@ using namespace sm100;
 constexpr int kDW = 256;                          // output rows per window (M of each MMA)
 constexpr int kDHalf = kDW / 2;                   // window rows each CTA holds (TMEM lanes)
 constexpr int kDN = 256;                          // most tokens per tile (N of each MMA)
-constexpr int kDStageK = 128;                     // k per stage: two 64-wide slabs
-constexpr int kDWBytes = kDHalf * kDStageK * 2;   // 32 KB of kept rows per stage at most
+constexpr int kDBoxK = 128;                       // k per copy: two 64-wide slabs
 constexpr int kDMaxXSlots = 8;                    // x slots (shared), at most
 constexpr int kDWSeq = 16;                        // W stages in flight, at most
 constexpr int kDConvWarp0 = 4, kDConvSets = 2, kDConvWarps = 4 * kDConvSets;   // a set per stage, in turn
@@ -70,18 +69,27 @@ constexpr uint64_t kDDrainLimitNs = 200000000ull;
 constexpr int kDRing = 224 * 1024;
 constexpr int kDSmem = kDRing + 1024;
 static_assert(kDSmem <= 226 * 1024, "shared memory budget");
-// x slots of a tile of n tokens (both CTAs): eight where the tile is small
-// (short MMAs: the copies' round trip is what they wait for), four of 32 KB at n = 256
-__host__ __device__ constexpr int d_x_slots(int n) { return n <= kDN / 2 ? kDMaxXSlots : kDMaxXSlots / 2; }
-// TMEM columns of D (n <= 64: two buffers), and the A slots the rest holds: a slot's
-// round trip (both CTAs' converters, the leader, the commit) is about 1.4 us, which
-// four slots hide at n = 256 (0.5 us of MMA a stage) and six about halve at small n
-__host__ __device__ constexpr uint32_t d_d_cols(int n) { return n <= kDN / 2 ? kDN / 2 : kDN; }
-__host__ __device__ constexpr uint32_t d_a_slots(int n) { return (512 - d_d_cols(n)) / (kDStageK / 2); }
+// A stage carries SK = 128 k, or 256 for tiles of up to 128 tokens (whose MMAs
+// are short: a stage then costs its hand-offs, about 0.35 us, however deep it is).
+// x slots of a tile of n tokens (both CTAs): eight where the tile is small and the
+// stage short, so that the copies' round trip is hidden
+__host__ __device__ constexpr int d_x_slots(int n, int sk) {
+  return sk == 256 ? (n <= 96 ? 4 : 3) : n <= kDN / 2 ? kDMaxXSlots : kDMaxXSlots / 2;
+}
+__host__ __device__ constexpr int d_w_ring(int n, int sk) { return kDRing - d_x_slots(n, sk) * (n / 2) * sk * 2; }
 // A W stage that would straddle the ring's end starts over at 0: with every
 // earlier stage released that asks for at most twice the largest stage.
-static_assert(kDRing - d_x_slots(kDN) * (kDN / 2) * kDStageK * 2 >= 2 * kDWBytes &&
-              kDRing - d_x_slots(kDN / 2) * (kDN / 4) * kDStageK * 2 >= 2 * kDWBytes, "two largest W stages fit the ring");
+constexpr bool d_ring_holds_two(int sk, int n_max) {
+  for (int n = 32; n <= n_max; n += 32)
+    if (d_w_ring(n, sk) < 2 * kDHalf * sk * 2) return false;
+  return true;
+}
+static_assert(d_ring_holds_two(128, kDN) && d_ring_holds_two(256, kDN / 2), "two largest W stages fit the ring");
+// TMEM columns of D (n <= 64: two buffers), and the A slots the rest holds: a slot's
+// round trip (both CTAs' converters, the leader, the commit) is about 1.4 us
+__host__ __device__ constexpr uint32_t d_d_cols(int n) { return n <= kDN / 2 ? kDN / 2 : kDN; }
+__host__ __device__ constexpr uint32_t d_a_slots(int n, int sk) { return (512 - d_d_cols(n)) / (uint32_t)(sk / 2); }
+static_assert(d_a_slots(kDN, 128) == 4 && d_a_slots(kDN / 2, 256) == 3, "A slots no more than x slots");
 
 struct DLayer {
   CUtensorMap xmap;          // x as (64, T, in/64) slabs, box 64 x N/2 x 2
@@ -231,7 +239,7 @@ __device__ __forceinline__ DRows d_rows(const DWalk<SQ>& W, int lane) {
 // kept block rows of a square item's column blocks in 128-row window win, R bits each
 template <int SQ>
 __device__ __forceinline__ uint64_t d_blocks(const DWalk<SQ>& W, int win, int lane) {
-  constexpr int kB = SQ > 0 ? kDStageK / SQ : 1, kR = SQ > 0 ? kDHalf / SQ : 1;
+  constexpr int kB = SQ > 0 ? kDBoxK / SQ : 1, kR = SQ > 0 ? kDHalf / SQ : 1;
   uint64_t v = 0;
   const int c = W.c0 + lane;
   if (W.valid() && c < W.L->G && win < W.L->nw) {
@@ -249,16 +257,17 @@ __device__ __forceinline__ uint32_t d_batch(const DWalk<SQ>& W, const DRows& r, 
 }
 
 // KW: item width (1 x KW groups; square groups: 128-column items); SQ: 0, or g
-// for square g x g groups
-template <int KW, int SQ>
+// for square g x g groups; SK: k per stage
+template <int KW, int SQ, int SK>
 __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_constant__ DParams P) {
-  constexpr int kStPer = KW / kDStageK;                   // stages per item
+  constexpr int kStPer = KW / SK;                         // stages per item
+  constexpr int kBoxes = SK / kDBoxK;                     // copies of x (1 x KW: of W) per stage
   constexpr int kRowK = SQ > 0 ? (SQ < 64 ? SQ : 64) : 64;   // columns of one kept-row piece in shared memory
   constexpr int kSub = 64 / kRowK;                        // row pieces per 64-wide slab
   constexpr int kPieces = kRowK / 8;                      // 16-byte pieces per row piece
-  constexpr int kBlk = 2 * kSub;                          // row pieces (square: column blocks) per stage
+  constexpr int kBlk = 2 * kSub;                          // row pieces (square: column blocks) per 128 k
   constexpr int kR = SQ > 0 ? kDHalf / SQ : 1;            // square: block rows per half window
-  static_assert(SQ == 0 || KW == kDStageK, "square items are one stage");
+  static_assert(KW % SK == 0 && SK % kDBoxK == 0 && (SQ == 0 || SK == kDBoxK), "items are whole stages");
   extern __shared__ uint8_t d_smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[kDMaxXSlots];  // leader: both CTAs' converters + both CTAs' x bytes
   __shared__ __align__(8) uint64_t done_bar[kDMaxXSlots];  // the stage's MMAs completed (both CTAs)
@@ -309,13 +318,13 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
   const int n_tiles = P.n_tiles;
   const int pair = (int)(blockIdx.x >> 1), n_pairs = (int)(gridDim.x >> 1);
   const int Nh = P.N / 2;                          // tokens of a tile each CTA loads
-  const uint32_t xs_n = (uint32_t)d_x_slots(P.N);  // x slots; full / done barriers in use
-  const uint32_t xs_bytes = (uint32_t)Nh * (kDStageK * 2);
-  const uint32_t w_ring = (uint32_t)kDRing - xs_n * xs_bytes;   // bytes of the W ring
+  const uint32_t xs_n = (uint32_t)d_x_slots(P.N, SK);  // x slots; full / done barriers in use
+  const uint32_t xs_bytes = (uint32_t)Nh * (SK * 2);
+  const uint32_t w_ring = (uint32_t)d_w_ring(P.N, SK);   // bytes of the W ring
   uint8_t* wsmem = smem + xs_n * xs_bytes;
   const uint32_t n_buf = P.N <= kDN / 4 ? 2u : 1u; // D buffers
   const uint32_t t_a = d_d_cols(P.N);              // first column of the A slots
-  const uint32_t a_n = d_a_slots(P.N);
+  const uint32_t a_n = d_a_slots(P.N, SK);
 
   if (P.inject_ns != 0 && pair == 0) {
     // test hook: before any copy or MMA is issued, a bounded wait on a word
@@ -364,8 +373,10 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
           }
           if (elect_one()) {
             if (rank == 0) mbar_arrive_expect_tx(&full_bar[s], 2u * xs_bytes);
-            tma_load_3d_pair(smem + s * xs_bytes, &L.xmap, mapa_shared(smem_u32(&full_bar[s]), 0), 0, tok0,
-                             c * (KW / 64) + 2 * st);
+#pragma unroll
+            for (int b = 0; b < kBoxes; ++b)
+              tma_load_3d_pair(smem + s * xs_bytes + b * (xs_bytes / kBoxes), &L.xmap,
+                               mapa_shared(smem_u32(&full_bar[s]), 0), 0, tok0, c * (KW / 64) + 2 * (st * kBoxes + b));
           }
           __syncwarp();
           if (++s == xs_n) {
@@ -477,9 +488,13 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
           const int start = w_start[i][0], h16 = ((int)w_n[i] + 15) / 16;
           for (int st = 0; st < kStPer && ok; ++st) {
             uint32_t off;
-            ok = slot((uint32_t)h16 * (16u * kDStageK * 2), off);
-            if (ok && h16 > 0 && elect_one())
-              tma_load_3d(wsmem + off, &L.wmap[h16 - 1], &wfull_bar[(k - 1) % kDWSeq], 0, start, 2 * st);
+            ok = slot((uint32_t)h16 * (16u * SK * 2), off);
+            if (ok && h16 > 0 && elect_one()) {
+#pragma unroll
+              for (int b = 0; b < kBoxes; ++b)
+                tma_load_3d(wsmem + off + b * h16 * (16 * kDBoxK * 2), &L.wmap[h16 - 1], &wfull_bar[(k - 1) % kDWSeq], 0,
+                            start, 2 * (st * kBoxes + b));
+            }
             __syncwarp();
           }
         }
@@ -529,12 +544,12 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
           break;
         }
         tc_fence_after();
-        const uint32_t a = tmem + t_a + as * (kDStageK / 2);
+        const uint32_t a = tmem + t_a + as * (SK / 2);
         const uint32_t b = x_lo + s * (xs_bytes >> 4);
         if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < kDStageK / 16; ++kk)
-            mma_bf16_ts_pair(d, a + 8 * kk, ((uint64_t)x_hi << 32) | (b + (kk >= 4 ? slab : 0u) + 2 * (kk & 3)), idesc,
+          for (int kk = 0; kk < SK / 16; ++kk)
+            mma_bf16_ts_pair(d, a + 8 * kk, ((uint64_t)x_hi << 32) | (b + (uint32_t)(kk >> 2) * slab + 2 * (kk & 3)), idesc,
                              (i == 0 && kk == 0) ? 0u : 1u);
           mma_commit_pair_mc(&done_bar[s], 0x3);
         }
@@ -575,9 +590,11 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
       if (k % kDConvSets == set) {
         const uint32_t e = k % kDWSeq;
         if (!d_wait_warp(&wfull_bar[e], (k / kDWSeq) & 1u, abort_flag, P.err)) return false;
-        uint32_t v[2][32];
-        {
-          const uint32_t base = smem_u32(wsmem) + hoff;
+        const uint32_t at = lane_addr + as * (SK / 2);
+#pragma unroll
+        for (int h = 0; h < kBoxes; ++h) {
+          uint32_t v[2][32];
+          const uint32_t base = smem_u32(wsmem) + hoff + (uint32_t)h * (bytes / kBoxes);
 #pragma unroll
           for (int b = 0; b < kBlk; ++b) {
             const uint32_t ro = (uint32_t)row[b] * (kRowK * 2);
@@ -613,14 +630,15 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
               o[3] = p[j].w;
             }
           }
+          __syncwarp();
+          if (h == kBoxes - 1 && lane == 0) mbar_arrive(&wempty_bar[e]);
+          if (h == 0) {
+            if (k >= a_n && !d_wait_warp(&done_bar[ds], dph, abort_flag, P.err)) return false;
+            tc_fence_after();
+          }
+          tmem_st_x32(at + 64 * h, v[0]);
+          tmem_st_x32(at + 64 * h + 32, v[1]);
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&wempty_bar[e]);
-        if (k >= a_n && !d_wait_warp(&done_bar[ds], dph, abort_flag, P.err)) return false;
-        tc_fence_after();
-        const uint32_t at = lane_addr + as * (kDStageK / 2);
-        tmem_st_x32(at, v[0]);
-        tmem_st_x32(at + 32, v[1]);
         tmem_wait_st();
         tc_fence_before();
         __syncwarp();
@@ -699,7 +717,7 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
           off[1] = slab;
 #pragma unroll
           for (int st = 0; st < kStPer; ++st)
-            if (ok) ok = stage(row, off, 2 * slab);
+            if (ok) ok = stage(row, off, kBoxes * 2 * slab);
         }
       }
     }
@@ -801,21 +819,21 @@ int d_sm_count() {
   return n;
 }
 
-template <int KW, int SQ>
+template <int KW, int SQ, int SK>
 cudaError_t d_set_attr() {
   static std::once_flag once;
   static cudaError_t err = cudaSuccess;
   std::call_once(once, []() {
-    err = cudaFuncSetAttribute(k_prefill_dense<KW, SQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDSmem);
+    err = cudaFuncSetAttribute(k_prefill_dense<KW, SQ, SK>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDSmem);
   });
   return err;
 }
 
-template <int KW, int SQ>
+template <int KW, int SQ, int SK>
 cudaError_t d_launch(const cudaLaunchConfig_t& cfg, const DParams& P) {
-  const cudaError_t e = d_set_attr<KW, SQ>();
+  const cudaError_t e = d_set_attr<KW, SQ, SK>();
   if (e != cudaSuccess) return e;
-  return cudaLaunchKernelEx(&cfg, k_prefill_dense<KW, SQ>, P);
+  return cudaLaunchKernelEx(&cfg, k_prefill_dense<KW, SQ, SK>, P);
 }
 
 }  // namespace
@@ -915,11 +933,12 @@ gs_status launch_prefill_dense(const void* const* xs, const gs_packed* const* ps
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    const cudaError_t e = sq == 16   ? d_launch<128, 16>(cfg, P)
-                          : sq == 32 ? d_launch<128, 32>(cfg, P)
-                          : sq == 64 ? d_launch<128, 64>(cfg, P)
-                          : kw == 256 ? d_launch<256, 0>(cfg, P)
-                                      : d_launch<128, 0>(cfg, P);
+    const cudaError_t e = sq == 16   ? d_launch<128, 16, 128>(cfg, P)
+                          : sq == 32 ? d_launch<128, 32, 128>(cfg, P)
+                          : sq == 64 ? d_launch<128, 64, 128>(cfg, P)
+                          : kw == 128 ? d_launch<128, 0, 128>(cfg, P)
+                          : tile_n <= kDN / 2 ? d_launch<256, 0, 256>(cfg, P)
+                                              : d_launch<256, 0, 128>(cfg, P);
     note_launch();
     if (e != cudaSuccess) return GS_ERR_CUDA;
   }
