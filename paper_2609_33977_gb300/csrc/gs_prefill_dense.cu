@@ -162,21 +162,32 @@ __device__ __forceinline__ uint32_t d_pack_bf16x2(float lo, float hi) {
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-// Whether item c of window w has MMAs: 1 x KW chunks with a kept row in the
-// window (square groups: every 128-column item)
-template <int SQ>
+// An item is kCh chunks (of KW columns; square: of 128) that share a stage, or one
+// chunk of one or more stages.
+template <int kCh>
+__device__ __forceinline__ int d_n_items(const DLayer& L) {
+  return kCh == 1 ? L.G : (L.G + kCh - 1) / kCh;
+}
+// Whether item c of window w has MMAs: 1 x KW items with a kept row in the
+// window (square groups: every item)
+template <int SQ, int kCh>
 __device__ __forceinline__ bool d_nonempty(const DLayer& L, int w, int c) {
-  if (c >= L.G) return false;
+  if (c >= d_n_items<kCh>(L)) return false;
   if constexpr (SQ > 0) return true;
-  const int32_t* wo = L.win_off + (int64_t)c * (L.nw + 1);
   const int lo = w * (kDW / kWin16), hi = min(lo + kDW / kWin16, L.nw);
-  return wo[hi] > wo[lo];
+  bool ne = false;
+#pragma unroll
+  for (int h = 0; h < kCh; ++h) {
+    const int32_t* wo = L.win_off + (int64_t)min(c * kCh + h, L.G - 1) * (L.nw + 1);
+    ne |= wo[hi] > wo[lo];
+  }
+  return ne;
 }
 // this lane's share of the number of items of window w (summed over the warp later)
-template <int SQ>
+template <int SQ, int kCh>
 __device__ __forceinline__ int d_count_part(const DLayer& L, int w, int lane) {
   int n = 0;
-  for (int c = lane; c < L.G; c += 32) n += d_nonempty<SQ>(L, w, c) ? 1 : 0;
+  for (int c = lane; c < d_n_items<kCh>(L); c += 32) n += d_nonempty<SQ, kCh>(L, w, c) ? 1 : 0;
   return n;
 }
 
@@ -195,7 +206,7 @@ __device__ __forceinline__ bool d_wait_warp(uint64_t* bar, uint32_t parity, vola
 // item c0 + l of the batch; what it loads for the next batch is in flight while
 // the warp works through this one.  (Loaded an item ahead instead, the lookups
 // queue behind the copies in flight: 1.0 us a stage instead of 0.5.)
-template <int SQ>
+template <int SQ, int kCh>
 struct DWalk {
   const DParams* P;
   int pair, n_pairs, ku, u, c0, w, m;
@@ -213,35 +224,40 @@ struct DWalk {
   __device__ __forceinline__ bool valid() const { return u >= 0; }
   __device__ __forceinline__ void next() {
     c0 += 32;
-    if (c0 >= L->G) {
+    if (c0 >= d_n_items<kCh>(*L)) {
       ++ku;
       unit();
     }
   }
 };
-// kept rows of a 1 x KW item: first packed row of the window's two halves and the end
+// kept rows of a 1 x KW item's chunks: first packed row of the window's two halves and the end
+template <int kCh>
 struct DRows {
-  int a, b, c;
+  int a[kCh], b[kCh], c[kCh];
 };
-template <int SQ>
-__device__ __forceinline__ DRows d_rows(const DWalk<SQ>& W, int lane) {
-  DRows r = {0, 0, 0};
-  const int c = W.c0 + lane;
-  if (W.valid() && c < W.L->G) {
-    const int nw = W.L->nw, lo = W.w * (kDW / kWin16);
-    const int32_t* wo = W.L->win_off + (int64_t)c * (nw + 1);
-    r.a = wo[lo];
-    r.b = wo[min(lo + kDHalf / kWin16, nw)];
-    r.c = wo[min(lo + kDW / kWin16, nw)];
+template <int SQ, int kCh>
+__device__ __forceinline__ DRows<kCh> d_rows(const DWalk<SQ, kCh>& W, int lane) {
+  DRows<kCh> r;
+#pragma unroll
+  for (int h = 0; h < kCh; ++h) {
+    r.a[h] = r.b[h] = r.c[h] = 0;
+    const int c = (W.c0 + lane) * kCh + h;
+    if (W.valid() && c < W.L->G) {
+      const int nw = W.L->nw, lo = W.w * (kDW / kWin16);
+      const int32_t* wo = W.L->win_off + (int64_t)c * (nw + 1);
+      r.a[h] = wo[lo];
+      r.b[h] = wo[min(lo + kDHalf / kWin16, nw)];
+      r.c[h] = wo[min(lo + kDW / kWin16, nw)];
+    }
   }
   return r;
 }
-// kept block rows of a square item's column blocks in 128-row window win, R bits each
-template <int SQ>
-__device__ __forceinline__ uint64_t d_blocks(const DWalk<SQ>& W, int win, int lane) {
+// kept block rows of the column blocks of a square item's chunk h in 128-row window win, R bits each
+template <int SQ, int kCh>
+__device__ __forceinline__ uint64_t d_blocks(const DWalk<SQ, kCh>& W, int h, int win, int lane) {
   constexpr int kB = SQ > 0 ? kDBoxK / SQ : 1, kR = SQ > 0 ? kDHalf / SQ : 1;
   uint64_t v = 0;
-  const int c = W.c0 + lane;
+  const int c = (W.c0 + lane) * kCh + h;
   if (W.valid() && c < W.L->G && win < W.L->nw) {
     const uint8_t* km = static_cast<const uint8_t*>(W.L->kmask) + (int64_t)c * kB * W.L->nw + win;
 #pragma unroll
@@ -250,32 +266,38 @@ __device__ __forceinline__ uint64_t d_blocks(const DWalk<SQ>& W, int win, int la
   return v;
 }
 // items of the batch that have MMAs (square groups: every item)
-template <int SQ>
-__device__ __forceinline__ uint32_t d_batch(const DWalk<SQ>& W, const DRows& r, int lane) {
-  if constexpr (SQ > 0) return __ballot_sync(0xffffffffu, W.c0 + lane < W.L->G);
-  return __ballot_sync(0xffffffffu, r.c > r.a);
+template <int SQ, int kCh>
+__device__ __forceinline__ uint32_t d_batch(const DWalk<SQ, kCh>& W, const DRows<kCh>& r, int lane) {
+  if constexpr (SQ > 0) return __ballot_sync(0xffffffffu, W.c0 + lane < d_n_items<kCh>(*W.L));
+  bool ne = false;
+#pragma unroll
+  for (int h = 0; h < kCh; ++h) ne |= r.c[h] > r.a[h];
+  return __ballot_sync(0xffffffffu, ne);
 }
 
-// KW: item width (1 x KW groups; square groups: 128-column items); SQ: 0, or g
-// for square g x g groups; SK: k per stage
+// KW: chunk width (1 x KW groups; square groups: 128); SQ: 0, or g for square
+// g x g groups; SK: k per stage
 template <int KW, int SQ, int SK>
 __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_constant__ DParams P) {
-  constexpr int kStPer = KW / SK;                         // stages per item
+  constexpr int kCh = KW < SK ? SK / KW : 1;              // chunks per item
+  constexpr int kItemK = KW * kCh;                        // columns per item
+  constexpr int kStPer = kItemK / SK;                     // stages per item
   constexpr int kBoxes = SK / kDBoxK;                     // copies of x (1 x KW: of W) per stage
   constexpr int kRowK = SQ > 0 ? (SQ < 64 ? SQ : 64) : 64;   // columns of one kept-row piece in shared memory
   constexpr int kSub = 64 / kRowK;                        // row pieces per 64-wide slab
   constexpr int kPieces = kRowK / 8;                      // 16-byte pieces per row piece
   constexpr int kBlk = 2 * kSub;                          // row pieces (square: column blocks) per 128 k
   constexpr int kR = SQ > 0 ? kDHalf / SQ : 1;            // square: block rows per half window
-  static_assert(KW % SK == 0 && SK % kDBoxK == 0 && (SQ == 0 || SK == kDBoxK), "items are whole stages");
+  static_assert(SK % kDBoxK == 0 && kItemK % SK == 0 && (kCh == 1 || KW == kDBoxK), "whole stages, a box a chunk");
   extern __shared__ uint8_t d_smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[kDMaxXSlots];  // leader: both CTAs' converters + both CTAs' x bytes
   __shared__ __align__(8) uint64_t done_bar[kDMaxXSlots];  // the stage's MMAs completed (both CTAs)
   __shared__ __align__(8) uint64_t wfull_bar[kDWSeq];      // local: W bytes landed
   __shared__ __align__(8) uint64_t wempty_bar[kDWSeq];     // local: the converters have read them
   __shared__ uint32_t w_end[kDWSeq];                       // virtual end of each W stage in the ring (W copy warp)
-  __shared__ int32_t w_start[32][SQ > 0 ? kBlk : 1];       // the batch's items: first packed row (square: tile) ...
-  __shared__ __align__(8) uint64_t w_n[32];                // ... and kept rows (square: kept block rows, d_blocks)
+  constexpr int kStarts = SQ > 0 ? kBlk : 1;
+  __shared__ int32_t w_start[32][kCh][kStarts];            // the batch's items: first packed row (square: tile) ...
+  __shared__ __align__(8) uint64_t w_n[32][kCh];           // ... and kept rows (square: kept block rows, d_blocks)
   __shared__ __align__(8) uint64_t afull_bar[2];          // D complete (both CTAs)
   __shared__ __align__(8) uint64_t aempty_bar[2];         // leader: D read by both CTAs' epilogues
   __shared__ __align__(8) uint64_t drain_bar;
@@ -355,8 +377,8 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
     uint32_t s = 0, ph = 1u;
     bool ok = true;
     asm volatile("griddepcontrol.wait;" ::: "memory");   // x may be the previous launch's output
-    DWalk<SQ> W(P, pair, n_pairs);
-    DRows nx = {0, 0, 0};
+    DWalk<SQ, kCh> W(P, pair, n_pairs);
+    DRows<kCh> nx = {};
     if constexpr (SQ == 0) nx = d_rows(W, lane);
     while (ok && W.valid()) {
       const DLayer& L = *W.L;
@@ -376,7 +398,7 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
 #pragma unroll
             for (int b = 0; b < kBoxes; ++b)
               tma_load_3d_pair(smem + s * xs_bytes + b * (xs_bytes / kBoxes), &L.xmap,
-                               mapa_shared(smem_u32(&full_bar[s]), 0), 0, tok0, c * (KW / 64) + 2 * (st * kBoxes + b));
+                               mapa_shared(smem_u32(&full_bar[s]), 0), 0, tok0, c * (kItemK / 64) + 2 * (st * kBoxes + b));
           }
           __syncwarp();
           if (++s == xs_n) {
@@ -423,48 +445,58 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
       ++k;
       return true;
     };
-    DWalk<SQ> W(P, pair, n_pairs);
+    DWalk<SQ, kCh> W(P, pair, n_pairs);
     if constexpr (SQ > 0) {
-      uint64_t mk_n;
-      int st_n[kBlk];
+      uint64_t mk_n[kCh];
+      int st_n[kCh][kBlk];
       auto load = [&]() {
         const int win = 2 * W.w + (int)rank;
-        mk_n = d_blocks(W, win, lane);
 #pragma unroll
-        for (int b = 0; b < kBlk; ++b) st_n[b] = 0;
-        if (W.valid() && W.c0 + lane < W.L->G && win < W.L->nw)
+        for (int h = 0; h < kCh; ++h) {
+          mk_n[h] = d_blocks(W, h, win, lane);
+          const int c = (W.c0 + lane) * kCh + h;
+          const bool in = W.valid() && c < W.L->G && win < W.L->nw;
 #pragma unroll
           for (int b = 0; b < kBlk; ++b)
-            st_n[b] = W.L->win_off[(int64_t)((W.c0 + lane) * kBlk + b) * (W.L->nw + 1) + win];
+            st_n[h][b] = in ? W.L->win_off[(int64_t)(c * kBlk + b) * (W.L->nw + 1) + win] : 0;
+        }
       };
       load();
       while (ok && W.valid()) {
         const DLayer& L = *W.L;
-        const int n_it = min(32, L.G - W.c0);
-        w_n[lane] = mk_n;
+        const int n_it = min(32, d_n_items<kCh>(L) - W.c0);
 #pragma unroll
-        for (int b = 0; b < kBlk; ++b) w_start[lane][b] = st_n[b];
+        for (int h = 0; h < kCh; ++h) {
+          w_n[lane][h] = mk_n[h];
+#pragma unroll
+          for (int b = 0; b < kBlk; ++b) w_start[lane][h][b] = st_n[h][b];
+        }
         W.next();
         load();
         __syncwarp();
         const uint16_t* tiles = L.tiles;
         for (int i = 0; i < n_it && ok; ++i) {
-          const uint64_t v = w_n[i];
-          uint32_t off;
-          ok = slot((uint32_t)__popcll(v) * (SQ * SQ * 2), off);
+          uint32_t off, n_all = 0;
+#pragma unroll
+          for (int h = 0; h < kCh; ++h) n_all += (uint32_t)__popcll(w_n[i][h]);
+          ok = slot(n_all * (SQ * SQ * 2), off);
           if (ok && elect_one()) {
             uint8_t* dst = wsmem + off;
             uint64_t* bar = &wfull_bar[(k - 1) % kDWSeq];
 #pragma unroll
-            for (int b = 0; b < kBlk; ++b) {
-              const int n = __popc((uint32_t)(v >> (b * kR)) & ((1u << kR) - 1u));
-              if (n > 0) {
-                const int start = w_start[i][b];
-                if constexpr (SQ < 64)
-                  bulk_g2s(dst, tiles + (int64_t)start * (SQ * SQ), (uint32_t)n * (SQ * SQ * 2), bar);
-                else
-                  tma_load_2d(dst, &L.wmap[n - 1], bar, 0, start * SQ);
-                dst += n * (SQ * SQ * 2);
+            for (int h = 0; h < kCh; ++h) {
+              const uint64_t v = w_n[i][h];
+#pragma unroll
+              for (int b = 0; b < kBlk; ++b) {
+                const int n = __popc((uint32_t)(v >> (b * kR)) & ((1u << kR) - 1u));
+                if (n > 0) {
+                  const int start = w_start[i][h][b];
+                  if constexpr (SQ < 64)
+                    bulk_g2s(dst, tiles + (int64_t)start * (SQ * SQ), (uint32_t)n * (SQ * SQ * 2), bar);
+                  else
+                    tma_load_2d(dst, &L.wmap[n - 1], bar, 0, start * SQ);
+                  dst += n * (SQ * SQ * 2);
+                }
               }
             }
           }
@@ -473,27 +505,39 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
         __syncwarp();   // every lane has read the batch
       }
     } else {
-      DRows nx = d_rows(W, lane);
+      DRows<kCh> nx = d_rows(W, lane);
       while (ok && W.valid()) {
         const DLayer& L = *W.L;
         uint32_t items = d_batch(W, nx, lane);
-        const int start_l = rank ? nx.b : nx.a;
-        w_start[lane][0] = start_l;
-        w_n[lane] = (uint64_t)((rank ? nx.c : nx.b) - start_l);
+#pragma unroll
+        for (int h = 0; h < kCh; ++h) {
+          const int start_l = rank ? nx.b[h] : nx.a[h];
+          w_start[lane][h][0] = start_l;
+          w_n[lane][h] = (uint64_t)((rank ? nx.c[h] : nx.b[h]) - start_l);
+        }
         W.next();
         nx = d_rows(W, lane);
         __syncwarp();
         for (; items && ok; items &= items - 1) {
           const int i = __ffs(items) - 1;
-          const int start = w_start[i][0], h16 = ((int)w_n[i] + 15) / 16;
+          uint32_t h16 = 0;   // 16-row steps of the item's chunks
+#pragma unroll
+          for (int h = 0; h < kCh; ++h) h16 += ((uint32_t)w_n[i][h] + 15) / 16;
           for (int st = 0; st < kStPer && ok; ++st) {
             uint32_t off;
-            ok = slot((uint32_t)h16 * (16u * SK * 2), off);
-            if (ok && h16 > 0 && elect_one()) {
+            ok = slot(h16 * (16u * (SK / kCh) * 2), off);
+            if (ok && elect_one()) {
+              uint8_t* dst = wsmem + off;
+              uint64_t* bar = &wfull_bar[(k - 1) % kDWSeq];
 #pragma unroll
-              for (int b = 0; b < kBoxes; ++b)
-                tma_load_3d(wsmem + off + b * h16 * (16 * kDBoxK * 2), &L.wmap[h16 - 1], &wfull_bar[(k - 1) % kDWSeq], 0,
-                            start, 2 * (st * kBoxes + b));
+              for (int b = 0; b < kBoxes; ++b) {
+                const int h = kCh > 1 ? b : 0;
+                const int hb = ((int)w_n[i][h] + 15) / 16;
+                if (hb > 0) {
+                  tma_load_3d(dst, &L.wmap[hb - 1], bar, 0, w_start[i][h][0], kCh > 1 ? 0 : 2 * (st * kBoxes + b));
+                  dst += hb * (16 * kDBoxK * 2);
+                }
+              }
             }
             __syncwarp();
           }
@@ -523,7 +567,7 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
     auto count = [&](int u) {
       if (u < 0) return 0;
       const DLayer& L = P.L[d_layer_of(P, u)];
-      return d_count_part<SQ>(L, (u - L.tile_begin) / L.n_m, lane);
+      return d_count_part<SQ, kCh>(L, (u - L.tile_begin) / L.n_m, lane);
     };
     int u = owner_tile(P.tl, n_tiles, pair, n_pairs, 0);
     part = count(u);
@@ -583,9 +627,10 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
     if (xs_n == a_n) ds = 0;
     uint32_t as = 0;                           // its A slot
     bool ok = true;
-    // one stage of `bytes` in the ring: row[b] = this lane's row in row piece b's
-    // compact block (-1: pruned), at off[b] from the stage's start
-    auto stage = [&](const int (&row)[kBlk], const uint32_t (&off)[kBlk], uint32_t bytes) {
+    // one stage of `bytes` in the ring; piece(h, b, row, off): this lane's row in the
+    // compact block of row piece b of 128-wide part h (-1: pruned), and the block's
+    // offset from the stage's start
+    auto stage = [&](auto&& piece, uint32_t bytes) {
       if (hoff + bytes > w_ring) hoff = 0;
       if (k % kDConvSets == set) {
         const uint32_t e = k % kDWSeq;
@@ -594,19 +639,22 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
 #pragma unroll
         for (int h = 0; h < kBoxes; ++h) {
           uint32_t v[2][32];
-          const uint32_t base = smem_u32(wsmem) + hoff + (uint32_t)h * (bytes / kBoxes);
+          const uint32_t base = smem_u32(wsmem) + hoff;
 #pragma unroll
           for (int b = 0; b < kBlk; ++b) {
-            const uint32_t ro = (uint32_t)row[b] * (kRowK * 2);
+            int row;
+            uint32_t off;
+            piece(h, b, row, off);
+            const uint32_t ro = (uint32_t)row * (kRowK * 2);
             // 16-byte piece j of a row is read from (64-wide rows, which TMA swizzled)
             // or at (plain rows) piece j ^ swz, which spreads eight rows over the banks
             const uint32_t swz = (ro >> 7) & (uint32_t)(kPieces - 1);
-            const uint32_t a = base + off[b] + ro;
+            const uint32_t a = base + off + ro;
             uint4 p[kPieces];
 #pragma unroll
             for (int j = 0; j < kPieces; ++j) {
               p[j] = make_uint4(0u, 0u, 0u, 0u);
-              if (row[b] >= 0) p[j] = lds128(a + (((uint32_t)j ^ swz) << 4));
+              if (row >= 0) p[j] = lds128(a + (((uint32_t)j ^ swz) << 4));
             }
             if constexpr (kRowK < 64) {
               // plain rows: piece j now lies in p[j ^ swz]
@@ -654,70 +702,97 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
       ++k;
       return true;
     };
-    DWalk<SQ> W(P, pair, n_pairs);
+    DWalk<SQ, kCh> W(P, pair, n_pairs);
     if constexpr (SQ > 0) {
       const int br = r / SQ;
-      uint64_t mk_n = d_blocks(W, 2 * W.w + (int)rank, lane);
-      while (ok && W.valid()) {
-        const uint64_t mk = mk_n;
-        const int n_it = min(32, W.L->G - W.c0);
-        W.next();
-        mk_n = d_blocks(W, 2 * W.w + (int)rank, lane);
-        for (int i = 0; i < n_it && ok; ++i) {
-          const uint64_t v = __shfl_sync(0xffffffffu, mk, i);
-          int row[kBlk];
-          uint32_t off[kBlk];
+      uint64_t mk_n[kCh];
+      auto load = [&]() {
 #pragma unroll
-          for (int b = 0; b < kBlk; ++b) {
-            const int at = b * kR;   // this block's bits
-            const uint32_t mb = (uint32_t)(v >> at) & ((1u << kR) - 1u);
-            row[b] = ((mb >> br) & 1u) ? (int)__popc(mb & ((1u << br) - 1u)) * SQ + r % SQ : -1;
-            off[b] = (uint32_t)__popcll(v & ((1ull << at) - 1ull)) * (SQ * SQ * 2);
+        for (int h = 0; h < kCh; ++h) mk_n[h] = d_blocks(W, h, 2 * W.w + (int)rank, lane);
+      };
+      load();
+      while (ok && W.valid()) {
+        uint64_t mk[kCh];
+#pragma unroll
+        for (int h = 0; h < kCh; ++h) mk[h] = mk_n[h];
+        const int n_it = min(32, d_n_items<kCh>(*W.L) - W.c0);
+        W.next();
+        load();
+        for (int i = 0; i < n_it && ok; ++i) {
+          uint64_t v[kCh];
+          uint32_t n_all = 0;
+#pragma unroll
+          for (int h = 0; h < kCh; ++h) {
+            v[h] = __shfl_sync(0xffffffffu, mk[h], i);
+            n_all += (uint32_t)__popcll(v[h]);
           }
-          ok = stage(row, off, (uint32_t)__popcll(v) * (SQ * SQ * 2));
+          ok = stage([&](int h, int b, int& row, uint32_t& off) {
+            const int at = b * kR;   // this block's bits
+            const uint32_t mb = (uint32_t)(v[h] >> at) & ((1u << kR) - 1u);
+            row = ((mb >> br) & 1u) ? (int)__popc(mb & ((1u << br) - 1u)) * SQ + r % SQ : -1;
+            off = (uint32_t)__popcll(v[h] & ((1ull << at) - 1ull));
+            for (int o = 0; o < h; ++o) off += (uint32_t)__popcll(v[o]);
+            off *= SQ * SQ * 2;
+          }, n_all * (SQ * SQ * 2));
         }
       }
     } else {
       // this warp's two 16-row windows in an item: kept masks, first packed row
-      uint32_t mk_n;
-      int wo_n;
+      uint32_t mk_n[kCh];
+      int wo_n[kCh];
       auto load = [&]() {
-        mk_n = 0;
-        wo_n = 0;
-        const int c = W.c0 + lane;
-        if (!W.valid() || c >= W.L->G) return;
-        const int nw = W.L->nw, b16 = W.w * (kDW / kWin16) + (int)rank * (kDHalf / kWin16) + 2 * q;
-        const uint16_t* km = static_cast<const uint16_t*>(W.L->kmask) + (int64_t)c * nw;
-        if (b16 < nw) {
-          mk_n = km[b16];
-          wo_n = W.L->win_off[(int64_t)c * (nw + 1) + b16];
+#pragma unroll
+        for (int h = 0; h < kCh; ++h) {
+          mk_n[h] = 0;
+          wo_n[h] = 0;
+          const int c = (W.c0 + lane) * kCh + h;
+          if (!W.valid() || c >= W.L->G) continue;
+          const int nw = W.L->nw, b16 = W.w * (kDW / kWin16) + (int)rank * (kDHalf / kWin16) + 2 * q;
+          const uint16_t* km = static_cast<const uint16_t*>(W.L->kmask) + (int64_t)c * nw;
+          if (b16 < nw) {
+            mk_n[h] = km[b16];
+            wo_n[h] = W.L->win_off[(int64_t)c * (nw + 1) + b16];
+          }
+          if (b16 + 1 < nw) mk_n[h] |= (uint32_t)km[b16 + 1] << 16;
         }
-        if (b16 + 1 < nw) mk_n |= (uint32_t)km[b16 + 1] << 16;
       };
-      DRows nx = d_rows(W, lane);
+      DRows<kCh> nx = d_rows(W, lane);
       load();
       while (ok && W.valid()) {
         uint32_t items = d_batch(W, nx, lane);
-        const int start_l = rank ? nx.b : nx.a, n_l = (rank ? nx.c : nx.b) - start_l;
-        const uint32_t mk_l = mk_n;
-        const int at_l = wo_n - start_l;
+        uint32_t mk_l[kCh];
+        int at_l[kCh];   // kept rows of the half window before this warp's rows | all of them << 16
+#pragma unroll
+        for (int h = 0; h < kCh; ++h) {
+          const int start_l = rank ? nx.b[h] : nx.a[h];
+          mk_l[h] = mk_n[h];
+          at_l[h] = ((wo_n[h] - start_l) & 0xffff) | (((rank ? nx.c[h] : nx.b[h]) - start_l) << 16);
+        }
         W.next();
         nx = d_rows(W, lane);
         load();
         for (; items && ok; items &= items - 1) {
           const int i = __ffs(items) - 1;
-          const uint32_t mk = __shfl_sync(0xffffffffu, mk_l, i);
-          const int n = __shfl_sync(0xffffffffu, n_l, i), at = __shfl_sync(0xffffffffu, at_l, i);
           // rows 32 q .. + 31 of the half window are consecutive bits, and consecutive in the slice
-          int row[kBlk];
-          uint32_t off[kBlk];
-          const uint32_t slab = (uint32_t)((n + 15) / 16) * (16 * 128);
-          row[0] = row[1] = ((mk >> lane) & 1u) ? at + (int)__popc(mk & ((1u << lane) - 1u)) : -1;
-          off[0] = 0;
-          off[1] = slab;
+          int row_c[kCh];
+          uint32_t slab[kCh], bytes = 0;
+#pragma unroll
+          for (int h = 0; h < kCh; ++h) {
+            const uint32_t mk = __shfl_sync(0xffffffffu, mk_l[h], i);
+            const int at = __shfl_sync(0xffffffffu, at_l[h], i);
+            row_c[h] = ((mk >> lane) & 1u) ? (at & 0xffff) + (int)__popc(mk & ((1u << lane) - 1u)) : -1;
+            slab[h] = (uint32_t)(((at >> 16) + 15) / 16) * (16 * 128);
+            bytes += slab[h] * (SK / kCh / 64);
+          }
 #pragma unroll
           for (int st = 0; st < kStPer; ++st)
-            if (ok) ok = stage(row, off, kBoxes * 2 * slab);
+            if (ok)
+              ok = stage([&](int h, int b, int& row, uint32_t& off) {
+                const int ch = kCh > 1 ? h : 0;
+                row = row_c[ch];
+                off = (uint32_t)b * slab[ch];
+                for (int o = 0; o < h; ++o) off += 2 * slab[kCh > 1 ? o : 0];
+              }, bytes);
         }
       }
     }
@@ -733,7 +808,7 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
       const DLayer& L = P.L[d_layer_of(P, u)];
       const int lt = u - L.tile_begin;
       const int m = lt % L.n_m, w = lt / L.n_m;
-      const bool any = __any_sync(0xffffffffu, d_count_part<SQ>(L, w, lane) > 0);   // else no MMA wrote D: zeros
+      const bool any = __any_sync(0xffffffffu, d_count_part<SQ, kCh>(L, w, lane) > 0);   // else no MMA wrote D: zeros
       const uint32_t buf = kb % n_buf;
       if (!d_wait_warp(&afull_bar[buf], (kb / n_buf) & 1u, abort_flag, P.err)) {
         ok = false;
@@ -933,12 +1008,12 @@ gs_status launch_prefill_dense(const void* const* xs, const gs_packed* const* ps
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
+    const bool deep = tile_n <= kDN / 2;   // 256-deep stages (16 x 16 groups: their lookups would not fit)
     const cudaError_t e = sq == 16   ? d_launch<128, 16, 128>(cfg, P)
-                          : sq == 32 ? d_launch<128, 32, 128>(cfg, P)
-                          : sq == 64 ? d_launch<128, 64, 128>(cfg, P)
-                          : kw == 128 ? d_launch<128, 0, 128>(cfg, P)
-                          : tile_n <= kDN / 2 ? d_launch<256, 0, 256>(cfg, P)
-                                              : d_launch<256, 0, 128>(cfg, P);
+                          : sq == 32 ? (deep ? d_launch<128, 32, 256>(cfg, P) : d_launch<128, 32, 128>(cfg, P))
+                          : sq == 64 ? (deep ? d_launch<128, 64, 256>(cfg, P) : d_launch<128, 64, 128>(cfg, P))
+                          : kw == 128 ? (deep ? d_launch<128, 0, 256>(cfg, P) : d_launch<128, 0, 128>(cfg, P))
+                                      : (deep ? d_launch<256, 0, 256>(cfg, P) : d_launch<256, 0, 128>(cfg, P));
     note_launch();
     if (e != cudaSuccess) return GS_ERR_CUDA;
   }
