@@ -335,7 +335,11 @@ static gs_status linear_impl(const void* x_dev, const gs_packed* p, int64_t T, v
   if (is_square(p)) return sq_linear_batched(&x_dev, &p, 1, T, &y_dev, s);   // one kernel family for every T
   if (algo == GS_ALGO_AUTO) {
     // the same per-layer choice as gs_linear_batched makes
-    if (T < kPrefillMinTokens) algo = GS_ALGO_DECODE;
+    if (T < kPrefillMinTokens) {
+      if (prefill_prefers_dense(p, T) && decode_prefers_dense(&p, 1, T))
+        return launch_prefill_dense(&x_dev, &p, 1, T, &y_dev, s, nullptr, true);
+      algo = GS_ALGO_DECODE;
+    }
     else if (prefill_prefers_dense(p, T)) algo = GS_ALGO_PREFILL_DENSE;
     else algo = p->G <= prefill_max_chunks() ? GS_ALGO_PREFILL : GS_ALGO_DECODE;
   }
@@ -448,6 +452,14 @@ gs_status gs_linear_batched(int32_t n, const void* const* xs_dev, const gs_packe
     }
     if (pp.empty()) return GS_OK;
     return launch_prefill_batched(xp.data(), pp.data(), (int)pp.size(), T, yp.data(), s);
+  }
+  if (decode_prefers_dense(ps, n, T)) {
+    std::vector<int> idx;
+    for (int i = 0; i < n; ++i) {
+      if (prefill_prefers_dense(ps[i], T)) idx.push_back(i);
+      else if (cudaMemsetAsync(ys_dev[i], 0, (size_t)T * (size_t)ps[i]->out * 2, s) != cudaSuccess) return GS_ERR_CUDA;
+    }
+    return launch_prefill_dense(xs_dev, ps, (int)idx.size(), T, ys_dev, s, idx.data(), true);
   }
   const int64_t blk = decode_max_tokens();
   std::vector<const void*> xb(n);

@@ -180,11 +180,14 @@ gs_status launch_prefill_batched(const void* const* xs, const gs_packed* const* 
                                  void* const* ys, cudaStream_t s);
 int prefill_max_chunks();
 // prefill_dense.cu: zero-filled windows (1 x 128 / 1 x 256 layers with kept groups)
-// (layers ps[idx[k]], k < n, when idx is given; else ps[0..n))
+// (layers ps[idx[k]], k < n, when idx is given; else ps[0..n)).  split: at T <= 16 units may be
+// split along the input, with the decode path's per-stream scratch (1 x KW layers).
 gs_status launch_prefill_dense(const void* const* xs, const gs_packed* const* ps, int n, int64_t T, void* const* ys,
-                               cudaStream_t s, const int* idx = nullptr);
+                               cudaStream_t s, const int* idx = nullptr, bool split = false);
 // whether the zero-filled kernel is the faster one for this layer and token count
 bool prefill_prefers_dense(const gs_packed* p, int64_t T);
+// whether a call of at most 16 tokens over these 1 x KW layers (one chunk width) takes it, split
+bool decode_prefers_dense(const gs_packed* const* ps, int n, int64_t T);
 
 // groups.cu: square g x g groups
 bool sq_shape_supported(int g_out, int g_in);

@@ -98,7 +98,9 @@ struct DLayer {
   const int32_t* win_off;    // 1 x KW: [G][nw16 + 1]; square: gwoff [in / g][nwin + 1]
   const void* kmask;         // 1 x KW: uint16 [G][nw16]; square: uint8 [in / g][nwin]
   uint16_t* y;
-  int32_t out, G, nw, n_m, tile_begin;   // G: chunks of KW columns (square: of 128); nw: 16-row (square: 128-row) windows
+  float* ws;                 // n_split > 1: [32-row blocks][n_split][32 rows][16 tokens] partial sums
+  int32_t* cnt;              // ... and arrival counters [32-row blocks] (zero between launches)
+  int32_t out, G, nw, n_m, n_split, tile_begin;   // G: chunks of KW columns (square: of 128); nw: 16-row (square: 128-row) windows
 };
 struct DParams {
   DLayer L[kDMaxLayers];
@@ -109,6 +111,12 @@ struct DParams {
 };
 static_assert(sizeof(DParams) <= 32764, "kernel parameter limit");
 
+// atomic add with acquire-release ordering at GPU scope; returns the old value
+__device__ __forceinline__ int d_atom_add_acq_rel(int32_t* p, int v) {
+  int old;
+  asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
+  return old;
+}
 __device__ __forceinline__ int d_layer_of(const DParams& P, int t) {
   int l = 0;
   while (l + 1 < P.n_layers && P.L[l + 1].tile_begin <= t) ++l;
@@ -183,11 +191,33 @@ __device__ __forceinline__ bool d_nonempty(const DLayer& L, int w, int c) {
   }
   return ne;
 }
-// this lane's share of the number of items of window w (summed over the warp later)
+// A unit: window w, token tile m, and items i0 .. i1 - 1 (part sp of n_split)
+struct DUnit {
+  int w, m, sp, i0, i1;
+};
+template <int kCh, bool kSplit>
+__device__ __forceinline__ DUnit d_unit(const DLayer& L, int u) {
+  DUnit U;
+  int lt = u - L.tile_begin;
+  U.m = lt % L.n_m;
+  U.w = lt / L.n_m;
+  U.sp = 0;
+  U.i0 = 0;
+  U.i1 = d_n_items<kCh>(L);
+  if constexpr (kSplit) {
+    const int n = U.i1;
+    U.sp = U.w % L.n_split;
+    U.w /= L.n_split;
+    U.i0 = U.sp * n / L.n_split;
+    U.i1 = (U.sp + 1) * n / L.n_split;
+  }
+  return U;
+}
+// this lane's share of the number of items of a unit that have MMAs (summed over the warp later)
 template <int SQ, int kCh>
-__device__ __forceinline__ int d_count_part(const DLayer& L, int w, int lane) {
+__device__ __forceinline__ int d_count_part(const DLayer& L, const DUnit& U, int lane) {
   int n = 0;
-  for (int c = lane; c < d_n_items<kCh>(L); c += 32) n += d_nonempty<SQ, kCh>(L, w, c) ? 1 : 0;
+  for (int c = U.i0 + lane; c < U.i1; c += 32) n += d_nonempty<SQ, kCh>(L, U.w, c) ? 1 : 0;
   return n;
 }
 
@@ -206,25 +236,28 @@ __device__ __forceinline__ bool d_wait_warp(uint64_t* bar, uint32_t parity, vola
 // item c0 + l of the batch; what it loads for the next batch is in flight while
 // the warp works through this one.  (Loaded an item ahead instead, the lookups
 // queue behind the copies in flight: 1.0 us a stage instead of 0.5.)
-template <int SQ, int kCh>
+template <int SQ, int kCh, bool kSplit>
 struct DWalk {
   const DParams* P;
-  int pair, n_pairs, ku, u, c0, w, m;
+  int pair, n_pairs, ku, u, c0, c1, w, m;   // c1: end of the unit's items
   const DLayer* L;
   __device__ __forceinline__ void unit() {
     u = owner_tile(P->tl, P->n_tiles, pair, n_pairs, ku);
-    c0 = 0;
     if (u < 0) return;
     L = &P->L[d_layer_of(*P, u)];
-    const int lt = u - L->tile_begin;
-    m = lt % L->n_m;
-    w = lt / L->n_m;
+    const DUnit U = d_unit<kCh, kSplit>(*L, u);
+    w = U.w;
+    m = U.m;
+    c0 = U.i0;
+    c1 = U.i1;
   }
+  // item c0 + lane is in the unit
+  __device__ __forceinline__ bool has(int lane) const { return u >= 0 && c0 + lane < c1; }
   __device__ __forceinline__ DWalk(const DParams& p, int pr, int n) : P(&p), pair(pr), n_pairs(n), ku(0) { unit(); }
   __device__ __forceinline__ bool valid() const { return u >= 0; }
   __device__ __forceinline__ void next() {
     c0 += 32;
-    if (c0 >= d_n_items<kCh>(*L)) {
+    if (c0 >= c1) {
       ++ku;
       unit();
     }
@@ -235,14 +268,14 @@ template <int kCh>
 struct DRows {
   int a[kCh], b[kCh], c[kCh];
 };
-template <int SQ, int kCh>
-__device__ __forceinline__ DRows<kCh> d_rows(const DWalk<SQ, kCh>& W, int lane) {
+template <int SQ, int kCh, bool kSplit>
+__device__ __forceinline__ DRows<kCh> d_rows(const DWalk<SQ, kCh, kSplit>& W, int lane) {
   DRows<kCh> r;
 #pragma unroll
   for (int h = 0; h < kCh; ++h) {
     r.a[h] = r.b[h] = r.c[h] = 0;
     const int c = (W.c0 + lane) * kCh + h;
-    if (W.valid() && c < W.L->G) {
+    if (W.has(lane) && c < W.L->G) {
       const int nw = W.L->nw, lo = W.w * (kDW / kWin16);
       const int32_t* wo = W.L->win_off + (int64_t)c * (nw + 1);
       r.a[h] = wo[lo];
@@ -253,12 +286,12 @@ __device__ __forceinline__ DRows<kCh> d_rows(const DWalk<SQ, kCh>& W, int lane) 
   return r;
 }
 // kept block rows of the column blocks of a square item's chunk h in 128-row window win, R bits each
-template <int SQ, int kCh>
-__device__ __forceinline__ uint64_t d_blocks(const DWalk<SQ, kCh>& W, int h, int win, int lane) {
+template <int SQ, int kCh, bool kSplit>
+__device__ __forceinline__ uint64_t d_blocks(const DWalk<SQ, kCh, kSplit>& W, int h, int win, int lane) {
   constexpr int kB = SQ > 0 ? kDBoxK / SQ : 1, kR = SQ > 0 ? kDHalf / SQ : 1;
   uint64_t v = 0;
   const int c = (W.c0 + lane) * kCh + h;
-  if (W.valid() && c < W.L->G && win < W.L->nw) {
+  if (W.has(lane) && c < W.L->G && win < W.L->nw) {
     const uint8_t* km = static_cast<const uint8_t*>(W.L->kmask) + (int64_t)c * kB * W.L->nw + win;
 #pragma unroll
     for (int b = 0; b < kB; ++b) v |= (uint64_t)km[(int64_t)b * W.L->nw] << (b * kR);
@@ -266,18 +299,57 @@ __device__ __forceinline__ uint64_t d_blocks(const DWalk<SQ, kCh>& W, int h, int
   return v;
 }
 // items of the batch that have MMAs (square groups: every item)
-template <int SQ, int kCh>
-__device__ __forceinline__ uint32_t d_batch(const DWalk<SQ, kCh>& W, const DRows<kCh>& r, int lane) {
-  if constexpr (SQ > 0) return __ballot_sync(0xffffffffu, W.c0 + lane < d_n_items<kCh>(*W.L));
+template <int SQ, int kCh, bool kSplit>
+__device__ __forceinline__ uint32_t d_batch(const DWalk<SQ, kCh, kSplit>& W, const DRows<kCh>& r, int lane) {
+  if constexpr (SQ > 0) return __ballot_sync(0xffffffffu, W.has(lane));
   bool ne = false;
 #pragma unroll
   for (int h = 0; h < kCh; ++h) ne |= r.c[h] > r.a[h];
   return __ballot_sync(0xffffffffu, ne);
 }
 
+// The last part of a 32-row block to arrive adds them all, in split order, and
+// writes y (part: this lane's row of split 0).
+__device__ __forceinline__ void d_reduce_parts(const DLayer& L, const float4* part, int row0, int lane, int T) {
+  if (lane == 0) L.cnt[row0 / 32] = 0;
+  uint16_t* yp = L.y + row0 + lane;
+  const bool in_row = row0 + lane < L.out;
+#pragma unroll 1
+  for (int c0 = 0; 4 * c0 < T; c0 += 2) {   // eight tokens, four splits' loads in flight
+    float4 acc[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+#pragma unroll 1
+    for (int s0 = 0; s0 < L.n_split; s0 += 4) {
+      float4 f[4][2];
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+          if (s0 + j < L.n_split && 4 * (c0 + c) < T) f[j][c] = __ldcg(part + (s0 + j) * 128 + c0 + c);
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+          if (s0 + j < L.n_split && 4 * (c0 + c) < T) {
+            acc[c].x += f[j][c].x;
+            acc[c].y += f[j][c].y;
+            acc[c].z += f[j][c].z;
+            acc[c].w += f[j][c].w;
+          }
+    }
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const float a[4] = {acc[c].x, acc[c].y, acc[c].z, acc[c].w};
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+        if (in_row && 4 * (c0 + c) + t < T)
+          yp[(int64_t)(4 * (c0 + c) + t) * L.out] = __bfloat16_as_ushort(__float2bfloat16_rn(a[t]));
+    }
+  }
+}
+
 // KW: chunk width (1 x KW groups; square groups: 128); SQ: 0, or g for square
-// g x g groups; SK: k per stage
-template <int KW, int SQ, int SK>
+// g x g groups; SK: k per stage; kSplit: layers may have several parts per window
+template <int KW, int SQ, int SK, bool kSplit>
 __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_constant__ DParams P) {
   constexpr int kCh = KW < SK ? SK / KW : 1;              // chunks per item
   constexpr int kItemK = KW * kCh;                        // columns per item
@@ -377,7 +449,7 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
     uint32_t s = 0, ph = 1u;
     bool ok = true;
     asm volatile("griddepcontrol.wait;" ::: "memory");   // x may be the previous launch's output
-    DWalk<SQ, kCh> W(P, pair, n_pairs);
+    DWalk<SQ, kCh, kSplit> W(P, pair, n_pairs);
     DRows<kCh> nx = {};
     if constexpr (SQ == 0) nx = d_rows(W, lane);
     while (ok && W.valid()) {
@@ -445,7 +517,7 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
       ++k;
       return true;
     };
-    DWalk<SQ, kCh> W(P, pair, n_pairs);
+    DWalk<SQ, kCh, kSplit> W(P, pair, n_pairs);
     if constexpr (SQ > 0) {
       uint64_t mk_n[kCh];
       int st_n[kCh][kBlk];
@@ -455,7 +527,7 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
         for (int h = 0; h < kCh; ++h) {
           mk_n[h] = d_blocks(W, h, win, lane);
           const int c = (W.c0 + lane) * kCh + h;
-          const bool in = W.valid() && c < W.L->G && win < W.L->nw;
+          const bool in = W.has(lane) && c < W.L->G && win < W.L->nw;
 #pragma unroll
           for (int b = 0; b < kBlk; ++b)
             st_n[h][b] = in ? W.L->win_off[(int64_t)(c * kBlk + b) * (W.L->nw + 1) + win] : 0;
@@ -464,7 +536,7 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
       load();
       while (ok && W.valid()) {
         const DLayer& L = *W.L;
-        const int n_it = min(32, d_n_items<kCh>(L) - W.c0);
+        const int n_it = min(32, W.c1 - W.c0);
 #pragma unroll
         for (int h = 0; h < kCh; ++h) {
           w_n[lane][h] = mk_n[h];
@@ -567,7 +639,7 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
     auto count = [&](int u) {
       if (u < 0) return 0;
       const DLayer& L = P.L[d_layer_of(P, u)];
-      return d_count_part<SQ, kCh>(L, (u - L.tile_begin) / L.n_m, lane);
+      return d_count_part<SQ, kCh>(L, d_unit<kCh, kSplit>(L, u), lane);
     };
     int u = owner_tile(P.tl, n_tiles, pair, n_pairs, 0);
     part = count(u);
@@ -702,7 +774,7 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
       ++k;
       return true;
     };
-    DWalk<SQ, kCh> W(P, pair, n_pairs);
+    DWalk<SQ, kCh, kSplit> W(P, pair, n_pairs);
     if constexpr (SQ > 0) {
       const int br = r / SQ;
       uint64_t mk_n[kCh];
@@ -715,7 +787,7 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
         uint64_t mk[kCh];
 #pragma unroll
         for (int h = 0; h < kCh; ++h) mk[h] = mk_n[h];
-        const int n_it = min(32, d_n_items<kCh>(*W.L) - W.c0);
+        const int n_it = min(32, W.c1 - W.c0);
         W.next();
         load();
         for (int i = 0; i < n_it && ok; ++i) {
@@ -746,7 +818,7 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
           mk_n[h] = 0;
           wo_n[h] = 0;
           const int c = (W.c0 + lane) * kCh + h;
-          if (!W.valid() || c >= W.L->G) continue;
+          if (!W.has(lane) || c >= W.L->G) continue;
           const int nw = W.L->nw, b16 = W.w * (kDW / kWin16) + (int)rank * (kDHalf / kWin16) + 2 * q;
           const uint16_t* km = static_cast<const uint16_t*>(W.L->kmask) + (int64_t)c * nw;
           if (b16 < nw) {
@@ -804,21 +876,65 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
     uint32_t kb = 0;
     bool ok = true;
     const uint32_t leader_empty = mapa_shared(smem_u32(aempty_bar), 0);
-    for (int ku = 0, u; ok && (u = owner_tile(P.tl, n_tiles, pair, n_pairs, ku)) >= 0; ++ku, ++kb) {
+    int part_n = 0;   // items of the next unit, counted while this one runs
+    auto count = [&](int v) {
+      if (v < 0) return 0;
+      const DLayer& L = P.L[d_layer_of(P, v)];
+      return d_count_part<SQ, kCh>(L, d_unit<kCh, kSplit>(L, v), lane);
+    };
+    int u_n = owner_tile(P.tl, n_tiles, pair, n_pairs, 0);
+    part_n = count(u_n);
+    for (int ku = 0; ok && u_n >= 0; ++ku, ++kb) {
+      const int u = u_n;
       const DLayer& L = P.L[d_layer_of(P, u)];
-      const int lt = u - L.tile_begin;
-      const int m = lt % L.n_m, w = lt / L.n_m;
-      const bool any = __any_sync(0xffffffffu, d_count_part<SQ, kCh>(L, w, lane) > 0);   // else no MMA wrote D: zeros
+      const DUnit U = d_unit<kCh, kSplit>(L, u);
+      const int m = U.m, w = U.w;
+      const bool any = __any_sync(0xffffffffu, part_n > 0);   // else no MMA wrote D: zeros
+      u_n = owner_tile(P.tl, n_tiles, pair, n_pairs, ku + 1);
+      part_n = count(u_n);
       const uint32_t buf = kb % n_buf;
       if (!d_wait_warp(&afull_bar[buf], (kb / n_buf) & 1u, abort_flag, P.err)) {
         ok = false;
         break;
       }
       tc_fence_after();
-      uint32_t pk[kDN / 4];   // this lane's row: pairs of tokens
+      if (kSplit && L.n_split > 1) {
+        // T <= 16: the first half of the warps holds every token of the tile
+        uint32_t v[16];
+        if (hh == 0) {
+          tmem_ld_x16(tmem + ((uint32_t)(32 * q) << 16) + buf * (kDN / 4), v);
+          tmem_wait_ld();
+          reg_fence(v);
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster_relaxed(leader_empty + 8u * buf);   // D may be overwritten
+        const int row0 = w * kDW + (int)rank * kDHalf + 32 * q;
+        if (hh == 0 && row0 < L.out) {
+          // a lane's row: 16 tokens, 64 bytes
+          float4* part = reinterpret_cast<float4*>(L.ws + (int64_t)(row0 / 32) * L.n_split * 512) + 4 * lane;   // split 0
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            if (4 * c < P.T) {
+              const float* f = reinterpret_cast<const float*>(v + 4 * c);
+              part[U.sp * 128 + c] = any ? make_float4(f[0], f[1], f[2], f[3]) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+          __syncwarp();
+          int old = 0;
+          if (lane == 0) old = d_atom_add_acq_rel(&L.cnt[row0 / 32], 1);
+          if (__shfl_sync(0xffffffffu, old, 0) == L.n_split - 1) {
+            __syncwarp();
+            d_reduce_parts(L, part, row0, lane, P.T);
+          }
+        }
+        __syncwarp();
+        continue;
+      }
+      constexpr int kNL = kSplit ? 1 : kDN / 32;   // most 16-token loads (T <= 16: one)
+      uint32_t pk[8 * kNL];   // this lane's row: pairs of tokens
       const uint32_t dcol = tmem + ((uint32_t)(32 * q) << 16) + buf * (kDN / 4) + (uint32_t)(hh * Nh);
 #pragma unroll
-      for (int i = 0; i < kDN / 32; ++i)
+      for (int i = 0; i < kNL; ++i)
         if (i < nl) {
           uint32_t v[16];
           tmem_ld_x16(dcol + 16 * i, v);
@@ -840,7 +956,7 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
         const bool in_row = (row & ~1) < L.out;
         uint16_t* yp = L.y + (int64_t)(tok0 + (lane & 1)) * L.out + (row & ~1);
 #pragma unroll
-        for (int i = 0; i < kDN / 32; ++i)
+        for (int i = 0; i < kNL; ++i)
           if (i < nl) {
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
@@ -853,7 +969,7 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
       } else if (row < L.out) {
         uint16_t* yp = L.y + (int64_t)tok0 * L.out + row;
 #pragma unroll
-        for (int i = 0; i < kDN / 32; ++i)
+        for (int i = 0; i < kNL; ++i)
           if (i < nl) {
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
@@ -894,24 +1010,72 @@ int d_sm_count() {
   return n;
 }
 
-template <int KW, int SQ, int SK>
+template <int KW, int SQ, int SK, bool kSplit>
 cudaError_t d_set_attr() {
   static std::once_flag once;
   static cudaError_t err = cudaSuccess;
   std::call_once(once, []() {
-    err = cudaFuncSetAttribute(k_prefill_dense<KW, SQ, SK>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDSmem);
+    err = cudaFuncSetAttribute(k_prefill_dense<KW, SQ, SK, kSplit>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDSmem);
   });
   return err;
 }
 
-template <int KW, int SQ, int SK>
+template <int KW, int SQ, int SK, bool kSplit = false>
 cudaError_t d_launch(const cudaLaunchConfig_t& cfg, const DParams& P) {
-  const cudaError_t e = d_set_attr<KW, SQ, SK>();
+  const cudaError_t e = d_set_attr<KW, SQ, SK, kSplit>();
   if (e != cudaSuccess) return e;
-  return cudaLaunchKernelEx(&cfg, k_prefill_dense<KW, SQ, SK>, P);
+  return cudaLaunchKernelEx(&cfg, k_prefill_dense<KW, SQ, SK, kSplit>, P);
 }
 
 }  // namespace
+
+// Parts per window of each layer of a launch of at most 16 tokens.  Whole windows
+// alone can be too few or too long to fill 76 CTA pairs: a 5120 x 13824 layer (20
+// windows of 54 items) took 35 us, 21 in three parts.  But a part costs what about
+// six items do (partial sums out and in, an atomic): 13824 x 5120 took 17 us whole
+// and 21 to 30 us in four parts, a 7B block 37 us whole and 43 us with its 43-item
+// windows in parts of ten.
+void d_plan_splits(const std::vector<int>& units, const std::vector<int>& items, const std::vector<int>& most,
+                   int owners, std::vector<int>& split) {
+  const int n = (int)units.size();
+  int64_t total = 0;
+  int longest = 0, n_units = 0;
+  bool same = true;
+  for (int i = 0; i < n; ++i) {
+    total += (int64_t)units[i] * items[i];
+    n_units += units[i];
+    longest = std::max(longest, items[i]);
+    same = same && items[i] == items[0];
+  }
+  split.assign(n, 1);
+  const auto set = [&](int i, int s) { split[i] = std::max(1, std::min(s, std::min(most[i], items[i]))); };
+  const int avg = (int)((total + owners - 1) / owners);
+  if (same || n_units < owners) {
+    // the parts per longest window that leave the least to the busiest pair
+    int best = 1, best_cost = 1 << 30;
+    for (int s = 1; s <= 16 && s <= longest; ++s) {
+      int parts = 0, len = 0;
+      for (int i = 0; i < n; ++i) {
+        const int si = std::max(1, (s * items[i] + longest - 1) / longest);
+        parts += units[i] * si;
+        len = std::max(len, (items[i] + si - 1) / si);
+      }
+      const int cost = (parts + owners - 1) / owners * (len + (s > 1 ? 6 : 2));
+      if (cost < best_cost) {
+        best_cost = cost;
+        best = s;
+      }
+    }
+    for (int i = 0; i < n; ++i) set(i, (best * items[i] + longest - 1) / longest);
+    return;
+  }
+  // several lengths: only where a long window by itself outlasts the mean pair
+  // (Qwen2.5-7B block, 74 items against a mean of 47: 50 -> 44 us)
+  if (10 * longest <= 13 * avg) return;
+  const int len = std::max(8, avg / 2);
+  for (int i = 0; i < n; ++i)
+    if (2 * items[i] > avg) set(i, (items[i] + len - 1) / len);
+}
 
 // Which 1 x KW layers take this kernel: all that have kept groups, in the whole
 // prefill regime.  Against the gathering kernel, d = 0.5, us per batched block:
@@ -924,8 +1088,22 @@ bool prefill_prefers_dense(const gs_packed* p, int64_t T) {
   return p->kept > 0 && p->g_out == 1 && (p->g_in == 128 || p->g_in == 256);
 }
 
+// Whether a call of at most 16 tokens over layers of one chunk width takes this
+// kernel (split) rather than the decode kernel: from 20 M weights in all.  Below,
+// the few parts of a window cost more than the decode kernel's finer units (graph
+// replays, us at T = 1 / 16, this kernel against decode: 1024 x 1024 6 / 10 against
+// 5 / 8, 4096 x 4096 10 / 13 against 8 / 11; above: 5120 x 5120 11 / 13 against
+// 12 / 20, 20000 x 1024 9 / 9 against 16 / 31, 7B block 37 / 38 against 38 / 47 and
+// with 1 x 128 groups 40 / 40 against 60 / 65, 13B block 54 / 55 against 56 / 67).
+bool decode_prefers_dense(const gs_packed* const* ps, int n, int64_t T) {
+  if (T > 16) return false;
+  int64_t weights = 0;
+  for (int i = 0; i < n; ++i) weights += ps[i]->out * ps[i]->in;
+  return weights >= 20000000;
+}
+
 gs_status launch_prefill_dense(const void* const* xs, const gs_packed* const* ps, int n, int64_t T, void* const* ys,
-                               cudaStream_t s, const int* idx) {
+                               cudaStream_t s, const int* idx, bool split) {
   if (T <= 0 || n <= 0) return GS_OK;
   std::vector<int> order(n);
   for (int i = 0; i < n; ++i) order[i] = idx ? idx[i] : i;
@@ -949,10 +1127,33 @@ gs_status launch_prefill_dense(const void* const* xs, const gs_packed* const* ps
     DParams P;
     std::memset(&P, 0, sizeof(P));
     int64_t tiles = 0;
+    const bool deep = tile_n <= kDN / 2 && sq != 16;   // 256-deep stages (16 x 16 groups: their lookups would not fit)
+    const int item_k = sq == 0 && kw == 256 ? 256 : deep ? 256 : 128;
+    std::vector<int> parts(nb, 1);
+    if (split && T <= 16 && !sq) {
+      std::vector<int> units(nb), items(nb), most(nb);
+      for (int k = 0; k < nb; ++k) {
+        const gs_packed* p = ps[order[b0 + k]];
+        units[k] = (int)((p->out + kDW - 1) / kDW);
+        items[k] = (int)((p->in + item_k - 1) / item_k);
+        most[k] = p->dec_nsplit_max;
+      }
+      d_plan_splits(units, items, most, (int)max_pairs, parts);
+    }
     for (int k = 0; k < nb; ++k) {
       const int i = order[b0 + k];
       const gs_packed* p = ps[i];
       DLayer& L = P.L[k];
+      L.n_split = parts[k];
+      if (L.n_split > 1) {
+        // partial sums and counters in the decode path's per-stream scratch: 1024 floats per
+        // 64-row block and split there too, and at least one counter per 32 rows
+        const DecSlot* slot = nullptr;
+        const gs_status st = decode_slot(p, s, &slot);
+        if (st != GS_OK) return st;
+        L.ws = slot->ws;
+        L.cnt = slot->cnt;
+      }
       if (!encode_tmap_slabs_bf16(&L.xmap, xs[i], (uint64_t)p->in, (uint64_t)T, (uint32_t)(tile_n / 2), 2))
         return GS_ERR_CUDA;
       L.tiles = p->tiles;
@@ -975,7 +1176,7 @@ gs_status launch_prefill_dense(const void* const* xs, const gs_packed* const* ps
       if (L.G > 32767) return GS_ERR_UNSUPPORTED;
       L.n_m = (int32_t)n_m;
       L.tile_begin = (int32_t)tiles;
-      tiles += (int64_t)L.n_m * ((p->out + kDW - 1) / kDW);
+      tiles += (int64_t)L.n_m * L.n_split * ((p->out + kDW - 1) / kDW);
     }
     if (tiles > INT32_MAX) return GS_ERR_UNSUPPORTED;
     P.n_layers = nb;
@@ -983,14 +1184,15 @@ gs_status launch_prefill_dense(const void* const* xs, const gs_packed* const* ps
     P.N = (int32_t)tile_n;
     P.n_tiles = (int32_t)tiles;
     P.err = err;
-    P.inject_ns = b0 == 0 ? take_injected_wait(GS_ALGO_PREFILL_DENSE) : 0;
+    P.inject_ns = b0 == 0 ? take_injected_wait(split && T <= 16 ? GS_ALGO_DECODE : GS_ALGO_PREFILL_DENSE) : 0;
     const int owners = (int)std::min<int64_t>(tiles, max_pairs);
     if (tiles <= kTileListMax) {
       // a unit's time follows its item count (one launch holds one chunk width)
       std::vector<int32_t> cost((size_t)tiles);
       for (int k = 0; k < nb; ++k) {
-        const int64_t nu = (int64_t)P.L[k].n_m * ((ps[order[b0 + k]]->out + kDW - 1) / kDW);
-        for (int64_t t = 0; t < nu; ++t) cost[(size_t)(P.L[k].tile_begin + t)] = P.L[k].G;
+        const int64_t nu = (int64_t)P.L[k].n_m * parts[k] * ((ps[order[b0 + k]]->out + kDW - 1) / kDW);
+        const int32_t c = (P.L[k].G + parts[k] - 1) / parts[k];
+        for (int64_t t = 0; t < nu; ++t) cost[(size_t)(P.L[k].tile_begin + t)] = c;
       }
       plan_tiles(cost, owners, P.tl);
     }
@@ -1008,8 +1210,10 @@ gs_status launch_prefill_dense(const void* const* xs, const gs_packed* const* ps
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    const bool deep = tile_n <= kDN / 2;   // 256-deep stages (16 x 16 groups: their lookups would not fit)
-    const cudaError_t e = sq == 16   ? d_launch<128, 16, 128>(cfg, P)
+    bool any_split = false;
+    for (int k = 0; k < nb; ++k) any_split |= parts[k] > 1;
+    const cudaError_t e = any_split  ? (kw == 128 ? d_launch<128, 0, 256, true>(cfg, P) : d_launch<256, 0, 256, true>(cfg, P))
+                          : sq == 16   ? d_launch<128, 16, 128>(cfg, P)
                           : sq == 32 ? (deep ? d_launch<128, 32, 256>(cfg, P) : d_launch<128, 32, 128>(cfg, P))
                           : sq == 64 ? (deep ? d_launch<128, 64, 256>(cfg, P) : d_launch<128, 64, 128>(cfg, P))
                           : kw == 128 ? (deep ? d_launch<128, 0, 256>(cfg, P) : d_launch<128, 0, 128>(cfg, P))

@@ -133,6 +133,40 @@ def test_prefill_dense_token_tiles(gs, go, gi, d):
     assert gs.device_status() == gs.GS_OK
 
 
+@pytest.mark.parametrize("gi", [256, 128])
+@pytest.mark.parametrize("out,inp", [(1301, 16384), (5130, 4096)])
+def test_few_tokens_large_layers(gs, gi, out, inp):
+    """Calls of at most 16 tokens over 20 M weights or more: the zero-filled kernel with windows split
+    along the input (odd and ragged rows, an empty chunk range, every token count class), twice on the
+    same scratch, alone and batched with a layer of another width and one without kept groups."""
+    import torch
+    Wb = wl.random_weight_bits(out, inp, seed=out)
+    B = wl.random_mask(out, inp // gi, 0.5, seed=out + 1)
+    B[256:512, :inp // gi // 2] = 0   # a window whose first parts are empty
+    W2 = wl.random_weight_bits(640, 2048, seed=out + 2)
+    B2 = wl.random_mask(640, 2048 // gi, 0.4, seed=out + 3)
+    p, p2, p0 = (gs.pack_groups(to_dev(w), torch.from_numpy(np.ascontiguousarray(b)).cuda(), 1, gi)
+                 for w, b in ((Wb, B), (W2, B2), (W2, np.zeros_like(B2))))
+    for T in (1, 3, 4, 5, 8, 9, 13, 16):
+        xb, xb2 = wl.random_activation_bits(T, inp, seed=T), wl.random_activation_bits(T, 2048, seed=T + 50)
+        ref = orc.linear(xb, Wb, B, 1, gi)
+        ref2 = orc.linear(xb2, W2, B2, 1, gi)
+        x, x2 = to_dev(xb), to_dev(xb2)
+        for y in (gs.linear(x, p), gs.linear(x, p)):
+            assert np.all(np.abs(to_f64(y) - ref[0]) <= 2.0 ** -7 * ref[1] + 1e-6), (out, inp, gi, T)
+        ys = [torch.full((T, o), float("nan"), dtype=torch.bfloat16, device="cuda") for o in (out, 640, 640)]
+        gs.linear_batched_into([x, x2, x2], [p, p2, p0], ys)
+        assert np.all(np.abs(to_f64(ys[0]) - ref[0]) <= 2.0 ** -7 * ref[1] + 1e-6), (out, inp, gi, T)
+        assert np.all(np.abs(to_f64(ys[1]) - ref2[0]) <= 2.0 ** -7 * ref2[1] + 1e-6), (out, inp, gi, T)
+        assert np.all(to_f64(ys[2]) == 0.0)
+    assert gs.device_status() == gs.GS_OK
+
+
+def to_f64(t):
+    from tests._gpu_util import bf16_to_f64
+    return bf16_to_f64(to_bits(t))
+
+
 @pytest.mark.parametrize("go,gi", [(1, 256), (1, 128), (32, 32)])
 def test_prefill_dense_large_ragged_layers(gs, go, gi):
     """Zero-filled kernel on ~10K-row layers at T ~ 1K (80+ units, more than one per CTA pair):
