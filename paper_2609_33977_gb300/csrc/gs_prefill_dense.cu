@@ -80,7 +80,7 @@ __host__ __device__ constexpr int d_w_ring(int n, int sk) { return kDRing - d_x_
 // A W stage that would straddle the ring's end starts over at 0: with every
 // earlier stage released that asks for at most twice the largest stage.
 constexpr bool d_ring_holds_two(int sk, int n_max) {
-  for (int n = 32; n <= n_max; n += 32)
+  for (int n = 32; n <= n_max; n += 16)
     if (d_w_ring(n, sk) < 2 * kDHalf * sk * 2) return false;
   return true;
 }
@@ -871,7 +871,7 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
   } else if (warp >= kDEpiWarp0) {
     // ------------------------------------------------------------ epilogue
     const int q = warp & 3, hh = (warp - kDEpiWarp0) >> 2;   // TMEM lane quarter, half of the tile's tokens
-    const int nl = P.N / 32;                                 // 16-token loads per warp
+    const int nl = (Nh + 15) / 16;                           // 16-token loads per warp (the last may hold 8 of its own)
     asm volatile("griddepcontrol.wait;" ::: "memory");       // the previous launch may still use y
     uint32_t kb = 0;
     bool ok = true;
@@ -962,7 +962,7 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
             for (int e = 0; e < 8; ++e) {
               const int t = 16 * i + 2 * e;
               const uint32_t o = __shfl_xor_sync(0xffffffffu, pk[8 * i + e], 1);
-              if (in_row && tok0 + t + (lane & 1) < P.T)
+              if (in_row && t < Nh && tok0 + t + (lane & 1) < P.T)
                 *reinterpret_cast<uint32_t*>(yp + (int64_t)t * L.out) = __byte_perm(pk[8 * i + e], o, sel);
             }
           }
@@ -974,8 +974,8 @@ __global__ void __launch_bounds__(kDThreads, 1) k_prefill_dense(const __grid_con
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
               const int t = 16 * i + 2 * e;
-              if (tok0 + t < P.T) yp[(int64_t)t * L.out] = (uint16_t)pk[8 * i + e];
-              if (tok0 + t + 1 < P.T) yp[(int64_t)(t + 1) * L.out] = (uint16_t)(pk[8 * i + e] >> 16);
+              if (t < Nh && tok0 + t < P.T) yp[(int64_t)t * L.out] = (uint16_t)pk[8 * i + e];
+              if (t < Nh && tok0 + t + 1 < P.T) yp[(int64_t)(t + 1) * L.out] = (uint16_t)(pk[8 * i + e] >> 16);
             }
           }
       }
@@ -1119,9 +1119,10 @@ gs_status launch_prefill_dense(const void* const* xs, const gs_packed* const* ps
   // most tensor work per unit (the widest input) first
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return ps[a]->in > ps[b]->in; });
   const int64_t max_pairs = d_sm_count() / 2;
-  // tiles of equal size, in whole 32 tokens (16 per CTA and epilogue load)
+  // tiles of equal size, in whole 16 tokens (swizzled 8-row groups of x in each CTA;
+  // T = 777 takes four of 208 where whole 32 would be 224), at least 32
   const int64_t n_m = (T + kDN - 1) / kDN;
-  const int64_t tile_n = ((T + n_m - 1) / n_m + 31) / 32 * 32;
+  const int64_t tile_n = std::max<int64_t>(32, ((T + n_m - 1) / n_m + 15) / 16 * 16);
   for (int b0 = 0; b0 < n; b0 += kDMaxLayers) {
     const int nb = std::min(kDMaxLayers, n - b0);
     DParams P;

@@ -113,7 +113,7 @@ def test_prefill_dense_parity(gs, out, inp, d, seed):
 @pytest.mark.parametrize("go,gi", [(1, 256), (1, 128), (16, 16), (32, 32), (64, 64)])
 @pytest.mark.parametrize("d", [0.05, 0.5, 1.0])
 def test_prefill_dense_token_tiles(gs, go, gi, d):
-    """Zero-filled kernel at the edges of its token tiles (32-token steps, one and two accumulator
+    """Zero-filled kernel at the edges of its token tiles (16-token steps, one and two accumulator
     buffers, one and two tiles), with odd and ragged row counts, stages of every size in its byte
     ring (wrapping at d = 1) and a half window without a kept row."""
     import torch
@@ -124,7 +124,7 @@ def test_prefill_dense_token_tiles(gs, go, gi, d):
         B = wl.random_mask(out // go, inp // gi, d, seed=out + gi + 1)
         B[128 // go:min(256, out) // go, ::3] = 0
         p = gs.pack_groups(to_dev(Wb), torch.from_numpy(np.ascontiguousarray(B, dtype=np.uint8)).cuda(), go, gi)
-        for T in (17, 32, 33, 64, 65, 97, 128, 129, 161, 256, 257, 290):
+        for T in (17, 32, 33, 48, 64, 65, 97, 112, 128, 129, 161, 208, 256, 257, 290, 353):
             xb = wl.random_activation_bits(T, inp, seed=T + gi)
             y = to_bits(gs.linear(to_dev(xb), p, algo=gs.ALGO_PREFILL_DENSE if go == 1 else gs.ALGO_AUTO))
             yr, A = orc.linear(xb, Wb, B, go, gi)
