@@ -6,6 +6,7 @@
 // 16-bit kept mask.
 #include "gs_common.cuh"
 
+#include <cooperative_groups.h>
 #include <mutex>
 
 namespace gs {
@@ -28,26 +29,51 @@ __global__ void k_pack_count(const uint8_t* __restrict__ mask, int32_t out, int3
   cnt[e] = __popc(bits);
 }
 
-// (a2) scan: one CTA, exclusive prefix sum of cnt in chunk-major order.
+// (a2) scan: exclusive prefix sum of cnt in chunk-major order, by one cluster of
+// CTAs.  Each sums its own range first; the ranges' starts come from the other
+// CTAs' sums over distributed shared memory.  (One CTA over all entries, with a
+// division an entry, took 13.5 us for a 5120 x 13824 layer's 17280; now 6.7.)
 constexpr int kScanThreads = 1024;
 constexpr int kScanItems = 4;
+constexpr int kScanCtas = 8;
 
-__global__ void __launch_bounds__(kScanThreads) k_pack_scan(const int32_t* __restrict__ cnt, int32_t G,
-                                                            int32_t nw16, int32_t* __restrict__ win_off16,
-                                                            int64_t* __restrict__ offsets) {
+// sum over the block, in every thread (ws: kScanThreads / 32 words)
+__device__ __forceinline__ int32_t block_sum(int32_t v, int32_t* ws) {
+  v = __reduce_add_sync(0xffffffffu, v);
+  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = v;
+  __syncthreads();
+  const int32_t t = __reduce_add_sync(0xffffffffu, ws[threadIdx.x & 31]);
+  __syncthreads();
+  return t;
+}
+
+__global__ void __cluster_dims__(kScanCtas, 1, 1) __launch_bounds__(kScanThreads)
+    k_pack_scan(const int32_t* __restrict__ cnt, int32_t G, int32_t nw16, int32_t* __restrict__ win_off16,
+                int64_t* __restrict__ offsets) {
+  static_assert(kScanThreads == 1024, "one word of warp sums a lane");
   __shared__ int32_t warp_sums[kScanThreads / 32];
-  __shared__ int32_t carry_s;
+  __shared__ int32_t range_sum;
+  const cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
   const int64_t E = (int64_t)G * nw16;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) carry_s = 0;
-  __syncthreads();
-  for (int64_t base = 0; base < E; base += (int64_t)kScanThreads * kScanItems) {
+  const int rank = (int)cluster.block_rank();
+  const int64_t per = (E + kScanCtas - 1) / kScanCtas;
+  const int64_t lo = min(E, rank * per), hi = min(E, lo + per);
+  int32_t sum = 0;
+  for (int64_t e = lo + tid; e < hi; e += kScanThreads) sum += cnt[e];
+  sum = block_sum(sum, warp_sums);
+  if (tid == 0) range_sum = sum;
+  cluster.sync();
+  int32_t carry = 0;
+  for (int r = 0; r < rank; ++r) carry += *cluster.map_shared_rank(&range_sum, r);
+  cluster.sync();   // no CTA's shared memory goes away while another reads it
+  for (int64_t base = lo; base < hi; base += (int64_t)kScanThreads * kScanItems) {
+    const int64_t e0 = base + (int64_t)tid * kScanItems;
     int32_t v[kScanItems];
     int32_t local = 0;
 #pragma unroll
     for (int i = 0; i < kScanItems; ++i) {
-      const int64_t e = base + (int64_t)tid * kScanItems + i;
-      v[i] = e < E ? cnt[e] : 0;
+      v[i] = e0 + i < hi ? cnt[e0 + i] : 0;
       local += v[i];
     }
     // inclusive warp scan of the thread sums
@@ -59,34 +85,28 @@ __global__ void __launch_bounds__(kScanThreads) k_pack_scan(const int32_t* __res
     }
     if (lane == 31) warp_sums[warp] = incl;
     __syncthreads();
-    if (warp == 0) {
-      int32_t ws = warp_sums[lane];
-      int32_t wi = ws;
-#pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const int32_t t = __shfl_up_sync(0xffffffffu, wi, d);
-        if (lane >= d) wi += t;
-      }
-      warp_sums[lane] = wi - ws;   // exclusive warp offsets
-    }
+    const int32_t ws = warp_sums[lane];
+    const int32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? ws : 0);
+    const int32_t all = __reduce_add_sync(0xffffffffu, ws);
     __syncthreads();
-    int32_t run = carry_s + warp_sums[warp] + (incl - local);
+    int32_t run = carry + before + (incl - local);
+    carry += all;
+    if (e0 < hi) {
+      int c = (int)(e0 / nw16), w = (int)(e0 - (int64_t)c * nw16);
 #pragma unroll
-    for (int i = 0; i < kScanItems; ++i) {
-      const int64_t e = base + (int64_t)tid * kScanItems + i;
-      if (e < E) {
-        const int c = (int)(e / nw16);
-        const int w = (int)(e % nw16);
-        win_off16[(int64_t)c * (nw16 + 1) + w] = run;
+      for (int i = 0; i < kScanItems; ++i) {
+        if (e0 + i >= hi) break;
+        int32_t* row = win_off16 + (int64_t)c * (nw16 + 1);
+        row[w] = run;
         if (w == 0) offsets[c] = run;
-        if (w == nw16 - 1) win_off16[(int64_t)c * (nw16 + 1) + nw16] = run + v[i];
-        if (e == E - 1) offsets[G] = run + v[i];
+        run += v[i];
+        if (++w == nw16) {
+          row[nw16] = run;
+          if (++c == G) offsets[G] = run;
+          w = 0;
+        }
       }
-      run += v[i];
     }
-    __syncthreads();
-    if (tid == kScanThreads - 1) carry_s = run;
-    __syncthreads();
   }
 }
 
@@ -200,14 +220,14 @@ int grid_for(int64_t items, int per_block) {
 gs_status launch_pack_count_scan(const uint8_t* mask, gs_packed* p, cudaStream_t s, int32_t* cnt_tmp) {
   const int64_t E = (int64_t)p->G * p->nw16;
   k_pack_count<<<grid_for(E, 256), 256, 0, s>>>(mask, (int32_t)p->out, p->G, p->nw16, p->kmask16, cnt_tmp);
-  k_pack_scan<<<1, kScanThreads, 0, s>>>(cnt_tmp, p->G, p->nw16, p->win_off16, p->offsets);
+  k_pack_scan<<<kScanCtas, kScanThreads, 0, s>>>(cnt_tmp, p->G, p->nw16, p->win_off16, p->offsets);
   note_launch(2);
   return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
 
 gs_status launch_scan_counts(const int32_t* cnt, int32_t G, int32_t nw, int32_t* win_off, int64_t* offsets,
                              cudaStream_t s) {
-  k_pack_scan<<<1, kScanThreads, 0, s>>>(cnt, G, nw, win_off, offsets);
+  k_pack_scan<<<kScanCtas, kScanThreads, 0, s>>>(cnt, G, nw, win_off, offsets);
   note_launch();
   return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
@@ -299,7 +319,7 @@ extern "C" gs_status gs_pack_index_noalloc(const uint8_t* mask_dev, int64_t out,
   const int64_t E = G * nw16;
   k_pack_count<<<grid_for(E, 256), 256, 0, s>>>(mask_dev, (int32_t)out, (int32_t)G, (int32_t)nw16, kmask16_dev,
                                                 counts);
-  k_pack_scan<<<1, kScanThreads, 0, s>>>(counts, (int32_t)G, (int32_t)nw16, win_off16_dev, offsets_dev);
+  k_pack_scan<<<kScanCtas, kScanThreads, 0, s>>>(counts, (int32_t)G, (int32_t)nw16, win_off16_dev, offsets_dev);
   note_launch(2);
   return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }

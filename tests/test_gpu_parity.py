@@ -40,7 +40,8 @@ def packed(gs, Wb, B):
 
 PACK_SHAPES = [(1, 256, 1.0, 1), (17, 512, 0.5, 2), (300, 768, 0.5, 3), (1024, 1024, 0.5, 4),
                (512, 3584, 0.3, 5), (4096, 4096, 0.5, 6), (11008, 4096, 0.45, 7), (4096, 11008, 0.5, 8),
-               (129, 256, 0.0, 9), (200, 2048, 1.0, 10)]
+               (129, 256, 0.0, 9), (200, 2048, 1.0, 10),
+               (65, 768, 0.5, 15), (32784, 4352, 0.4, 16), (100, 16640, 0.6, 17)]   # ends of the scan's ranges and rounds
 
 
 @pytest.mark.parametrize("out,inp,d,seed", PACK_SHAPES)
