@@ -204,6 +204,10 @@ inline bool is_square(const gs_packed* p) { return p->g_out > 1; }
 // train.cu: Gumbel-Sigmoid sample and straight-through backward (Sec. 2.2)
 gs_status launch_gumbel(const float* logits, const float* noise, int64_t n, float tau, uint8_t* mask, float* dsdl,
                         int64_t* kept, cudaStream_t s);
+// group_grad.cu: the logit gradient in one pass over dy, x and W (dy^T x stays on chip), where it applies
+bool group_grad_fused(const void* x, const void* W, const gs_packed* p, const void* dy, int64_t T);
+gs_status launch_group_grad_fused(const void* x, const void* W, const gs_packed* p, const void* dy, int64_t T,
+                                  const float* dsdl, float* dlogits, int sm_count, cudaStream_t s);
 size_t backward_workspace_bytes(const gs_packed* p, bool want_dx);
 gs_status launch_backward(const void* x, const void* W, const gs_packed* p, const void* dy, int64_t T,
                           const float* dsdl, float* dlogits, void* dx, void* ws, cudaStream_t s);

@@ -123,16 +123,6 @@ __device__ __forceinline__ int d_layer_of(const DParams& P, int t) {
   return l;
 }
 
-// true in one lane of a converged warp (the same one each time)
-__device__ __forceinline__ bool elect_one() {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "elect.sync _|p, 0xffffffff;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(r));
-  return r != 0;
-}
 // D (M = 256: this CTA's 128 lanes and the peer's) (+)= A (TMEM, the same lanes
 // and columns in both CTAs) * B^T (N rows, half in each CTA's shared memory)
 __device__ __forceinline__ void mma_bf16_ts_pair(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,

@@ -244,6 +244,11 @@ gs_status launch_backward(const void* x, const void* W, const gs_packed* p, cons
                           const float* dsdl, float* dlogits, void* dx, void* ws, cudaStream_t s) {
   const int64_t out = p->out, in = p->in;
   float* D = static_cast<float*>(ws);
+  const bool fused = group_grad_fused(x, W, p, dy, T);
+  if (fused) {
+    const gs_status st = launch_group_grad_fused(x, W, p, dy, T, dsdl, dlogits, sm_count_train(), s);
+    if (st != GS_OK || !dx) return st;
+  }
   {
     std::lock_guard<std::mutex> lk(g_blas_mu);
     cublasHandle_t h = nullptr;
@@ -254,7 +259,7 @@ gs_status launch_backward(const void* x, const void* W, const gs_packed* p, cons
     // D [out][in] = dy^T x.  In cuBLAS's column-major terms D is (in x out) =
     // A (in x T) * B (T x out): x row-major [T][in] is A as stored; dy
     // row-major [T][out] is (out x T) as stored, so B is it transposed.
-    if (cublasGemmEx(h, CUBLAS_OP_N, CUBLAS_OP_T, (int)in, (int)out, (int)T, &one, x, CUDA_R_16BF, (int)in, dy,
+    if (!fused && cublasGemmEx(h, CUBLAS_OP_N, CUBLAS_OP_T, (int)in, (int)out, (int)T, &one, x, CUDA_R_16BF, (int)in, dy,
                      CUDA_R_16BF, (int)out, &zero, D, CUDA_R_32F, (int)in, CUBLAS_COMPUTE_32F,
                      CUBLAS_GEMM_DEFAULT) != CUBLAS_STATUS_SUCCESS)
       return GS_ERR_CUDA;
@@ -271,6 +276,7 @@ gs_status launch_backward(const void* x, const void* W, const gs_packed* p, cons
         return GS_ERR_CUDA;
     }
   }
+  if (fused) return GS_OK;
   const int64_t groups = (int64_t)(out / p->g_out) * (in / p->g_in);
   int64_t blocks = (groups + 7) / 8;
   if (blocks > (1 << 20)) blocks = 1 << 20;

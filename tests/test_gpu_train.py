@@ -115,6 +115,16 @@ def test_straight_through_backward(gs, g_out, g_in, T):
     backward_case(gs, 256, 512, g_out, g_in, T, seed=10 * T + g_in)
 
 
+@pytest.mark.parametrize("out,inp,g_in", [(64, 256, 256), (320, 1280, 256), (448, 1152, 128), (1000, 768, 256),
+                                          (5120, 2304, 256)])
+@pytest.mark.parametrize("T", [1, 63, 129])
+def test_backward_at_the_edges_of_the_one_pass_kernel(gs, out, inp, g_in, T):
+    """Row groups: ragged row windows, column tiles and token stages, several units per CTA pair (5120 x
+    2304: 180), and a row count (1000) that takes the two-pass route."""
+    backward_case(gs, out, inp, 1, g_in, T, seed=out + T, want_dx=out < 1000)
+    assert gs.device_status() == gs.GS_OK
+
+
 def test_backward_at_a_block_shape_without_dx(gs):
     backward_case(gs, 4096, 11008, 1, 256, 128, seed=77, want_dx=False)
     assert gs.device_status() == gs.GS_OK
