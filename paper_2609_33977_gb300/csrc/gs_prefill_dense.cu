@@ -1178,11 +1178,19 @@ gs_status launch_prefill_dense(const void* const* xs, const gs_packed* const* ps
     P.inject_ns = b0 == 0 ? take_injected_wait(split && T <= 16 ? GS_ALGO_DECODE : GS_ALGO_PREFILL_DENSE) : 0;
     const int owners = (int)std::min<int64_t>(tiles, max_pairs);
     if (tiles <= kTileListMax) {
-      // a unit's time follows its item count (one launch holds one chunk width)
+      // A unit's time follows its item count (one launch holds one chunk width) and, at
+      // 17 to 128 tokens, the kept rows each item brings (7B block at d = 0.3 / 0.5 / 0.7:
+      // 40 / 49 / 66 us at T = 128): about 1/4 + density an item.  A 13B block of mixed
+      // densities takes 73 -> 70 us so; at 16 tokens or fewer the same weights cost 2 to
+      // 12 %, above 128 tokens (117 / 121 us at T = 512, d = 0.3 / 0.5) they change nothing.
+      const bool by_kept = T > 16 && tile_n <= kDN / 2;
       std::vector<int32_t> cost((size_t)tiles);
       for (int k = 0; k < nb; ++k) {
         const int64_t nu = (int64_t)P.L[k].n_m * parts[k] * ((ps[order[b0 + k]]->out + kDW - 1) / kDW);
-        const int32_t c = (P.L[k].G + parts[k] - 1) / parts[k];
+        const gs_packed* p = ps[order[b0 + k]];
+        const double d = (double)p->kept * p->g_out * p->g_in / ((double)p->out * (double)p->in);
+        const int32_t items = (P.L[k].G + parts[k] - 1) / parts[k];
+        const int32_t c = by_kept ? (int32_t)(64.0 * items * (0.25 + d)) + 1 : items;
         for (int64_t t = 0; t < nu; ++t) cost[(size_t)(P.L[k].tile_begin + t)] = c;
       }
       plan_tiles(cost, owners, P.tl);
