@@ -1085,10 +1085,14 @@ bool prefill_prefers_dense(const gs_packed* p, int64_t T) {
 // 5 / 8, 4096 x 4096 10 / 13 against 8 / 11; above: 5120 x 5120 11 / 13 against
 // 12 / 20, 20000 x 1024 9 / 9 against 16 / 31, 7B block 37 / 38 against 38 / 47 and
 // with 1 x 128 groups 40 / 40 against 60 / 65, 13B block 54 / 55 against 56 / 67).
+// At one or two tokens the decode kernel streams a batch of 1 x 256 layers as fast up to
+// about 250 M weights (7B block 40.5 us a call against 39.5, Qwen2.5-7B 44 / 43 as graph
+// replays; 13B block 61 against 56) and its launch is prepared 5 us sooner on the host.
 bool decode_prefers_dense(const gs_packed* const* ps, int n, int64_t T) {
   if (T > 16) return false;
   int64_t weights = 0;
   for (int i = 0; i < n; ++i) weights += ps[i]->out * ps[i]->in;
+  if (T <= 2 && n > 1 && ps[0]->g_in == 256) return weights >= 250000000;
   return weights >= 20000000;
 }
 
