@@ -1067,6 +1067,47 @@ void d_plan_splits(const std::vector<int>& units, const std::vector<int>& items,
     if (2 * items[i] > avg) set(i, (items[i] + len - 1) / len);
 }
 
+// Tokens of each of n_m tiles of equal size: whole 16 tokens (swizzled 8-row groups of
+// x in each CTA; T = 777 takes four of 208 where whole 32 would be 224), at least 32.
+int64_t d_tile_tokens(int64_t T, int64_t n_m) { return std::max<int64_t>(32, ((T + n_m - 1) / n_m + 15) / 16 * 16); }
+
+// Token tiles of a launch: as few as 256 tokens each allow, or more and narrower ones
+// where those leave CTA pairs without a unit.  Estimated time: the busiest pair's
+// 256-column items times what one takes at n tokens (measured, ns: about 540 + 1.6 n
+// with 256-deep stages, up to 128 tokens; 4.4 n, at least 1000, above).  Narrower tiles
+// change no result: a row's products are added in the same order.  From three units a
+// pair on, or one with layers of several widths, the wide tiles stay (a Qwen2.5-7B block at
+// T = 200 took 84 us in two tiles of 112 and 78 in one).  Layers alone, us as graph replays: 4096 x 4096 at T = 256
+// 25 -> 16, 5120 x 13824 at T = 256 / 777 67 / 103 -> 42 / 80, 3000 x 12032 (1 x 128) at
+// T = 512 59 -> 41, 4096 x 11008 (64x64) at T = 512 52 -> 38; 16x16 groups, whose stages
+// are always 128 deep, 65 -> 66.
+int64_t d_token_tiles(const std::vector<int64_t>& units, const std::vector<int64_t>& items, int64_t T, int64_t owners,
+                      bool deep) {
+  const int64_t least = (T + kDN - 1) / kDN;
+  int64_t n_units = 0, total = 0, longest = 0;
+  for (size_t i = 0; i < units.size(); ++i) {
+    n_units += units[i];
+    total += units[i] * items[i];
+    longest = std::max(longest, items[i]);
+  }
+  const bool same = total == n_units * longest;
+  if (!deep || T <= kDN / 2 || n_units * least >= (same ? 3 : 1) * owners) return least;
+  int64_t best = least;
+  double best_cost = 0.0;
+  for (int64_t m = least; m <= 8 * least && (m == least || n_units * m <= 6 * owners); ++m) {
+    const int64_t n = d_tile_tokens(T, m);
+    const double item = n <= kDN / 2 ? 540.0 + 1.6 * (double)n : std::max(1000.0, 4.4 * (double)n);
+    const int64_t rounds = (n_units * m + owners - 1) / owners;
+    const int64_t busiest = same ? rounds * longest : std::max(longest * (rounds > 1 ? 2 : 1), (total * m + owners - 1) / owners);
+    const double cost = (double)busiest * item;
+    if (m == least || cost < 0.95 * best_cost) {
+      best_cost = cost;
+      best = m;
+    }
+  }
+  return best;
+}
+
 // Which 1 x KW layers take this kernel: all that have kept groups, in the whole
 // prefill regime.  Against the gathering kernel, d = 0.5, us per batched block:
 // 13B 1 x 256 at T = 17 / 128 / 256 / 512 71 / 76 / 93 / 168 against 92 / 98 / 173 / 294;
@@ -1113,15 +1154,21 @@ gs_status launch_prefill_dense(const void* const* xs, const gs_packed* const* ps
   // most tensor work per unit (the widest input) first
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return ps[a]->in > ps[b]->in; });
   const int64_t max_pairs = d_sm_count() / 2;
-  // tiles of equal size, in whole 16 tokens (swizzled 8-row groups of x in each CTA;
-  // T = 777 takes four of 208 where whole 32 would be 224), at least 32
-  const int64_t n_m = (T + kDN - 1) / kDN;
-  const int64_t tile_n = std::max<int64_t>(32, ((T + n_m - 1) / n_m + 15) / 16 * 16);
   for (int b0 = 0; b0 < n; b0 += kDMaxLayers) {
     const int nb = std::min(kDMaxLayers, n - b0);
     DParams P;
     std::memset(&P, 0, sizeof(P));
     int64_t tiles = 0;
+    int64_t n_m = (T + kDN - 1) / kDN;
+    {
+      std::vector<int64_t> units(nb), items(nb);
+      for (int k = 0; k < nb; ++k) {
+        units[k] = (ps[order[b0 + k]]->out + kDW - 1) / kDW;
+        items[k] = (ps[order[b0 + k]]->in + 255) / 256;
+      }
+      n_m = d_token_tiles(units, items, T, max_pairs, sq != 16);
+    }
+    const int64_t tile_n = d_tile_tokens(T, n_m);
     const bool deep = tile_n <= kDN / 2 && sq != 16;   // 256-deep stages (16 x 16 groups: their lookups would not fit)
     const int item_k = sq == 0 && kw == 256 ? 256 : deep ? 256 : 128;
     std::vector<int> parts(nb, 1);
