@@ -125,6 +125,22 @@ void handles_used(const gs_packed* const* ps, int n, cudaStream_t s) {
   }
 }
 
+bool may_overlap(const gs_packed* p, cudaStream_t s) {
+  // any other stream is ordered after packing by an event, a full dependency (the
+  // legacy stream has two names)
+  const auto one_name = [](void* x) { return x == static_cast<void*>(cudaStreamLegacy) ? nullptr : x; };
+  if (one_name(static_cast<void*>(s)) != one_name(p->pack_stream)) return true;
+  int32_t* fresh = const_cast<int32_t*>(&p->fresh);
+  if (!__atomic_load_n(fresh, __ATOMIC_ACQUIRE)) return true;
+  if (s == cudaStreamPerThread) return false;   // another stream in every thread
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  const cudaError_t e = cudaStreamIsCapturing(s, &st);
+  if (e != cudaSuccess) cudaGetLastError();
+  // a captured launch does not run now: the next one on the stream may still follow packing
+  if (e == cudaSuccess && st == cudaStreamCaptureStatusNone) __atomic_store_n(fresh, 0, __ATOMIC_RELEASE);
+  return false;
+}
+
 void handle_on_stream(gs_packed* p, cudaStream_t s) {
   p->pack_stream = static_cast<void*>(s);
   p->tag = pool_tag(p->device, s);
@@ -257,6 +273,7 @@ static gs_status pack_rows(const void* W_dev, const uint8_t* mask_dev, int64_t o
   if ((st = launch_pack_compact(W_dev, p, s)) != GS_OK) goto fail;
   if ((st = decode_prepare(p, s)) != GS_OK) goto fail;
   if ((st = prefill_prepare_weight_maps(p)) != GS_OK) goto fail;
+  __atomic_store_n(&p->fresh, 1, __ATOMIC_RELEASE);
   *handle = p;
   return GS_OK;
 
@@ -310,6 +327,7 @@ gs_status gs_pack_groups(const void* W_dev, const uint8_t* mask_dev, int64_t out
     delete p;
     return st;
   }
+  __atomic_store_n(&p->fresh, 1, __ATOMIC_RELEASE);
   *handle = p;
   return GS_OK;
 }

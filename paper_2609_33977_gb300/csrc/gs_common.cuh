@@ -54,6 +54,7 @@ struct gs_packed {
   int32_t nbufs;
   gs::PoolTag tag;
   void* pack_stream;   // cudaStream_t, compared only
+  int32_t fresh;       // atomic: no launch has followed packing on its stream yet (see may_overlap)
   int32_t shared;      // atomic: used on another stream than gs_pack's, or captured into a graph
   int64_t out, in;
   int32_t G;          // in / 256
@@ -131,6 +132,11 @@ void handle_free(gs_packed* p, const void* ptr);   // one of them, before the ha
 void handle_on_stream(gs_packed* p, cudaStream_t s);
 // notes that work using the handles is queued on s (before every call's first launch)
 void handles_used(const gs_packed* const* ps, int n, cudaStream_t s);
+// Whether a launch on s may use programmatic dependent launch.  The decode and
+// zero-filled kernels read weights and their index before they wait for the launch
+// before them, which is only sound while that launch is not the packing itself: a
+// handle's first launch on its pack stream is an ordinary one.
+bool may_overlap(const gs_packed* p, cudaStream_t s);
 // waits for s and reads the kept-group count into p->kept
 gs_status read_kept(gs_packed* p, const int64_t* kept_dev, cudaStream_t s);
 // pool.cu: idle device buffers of released handles

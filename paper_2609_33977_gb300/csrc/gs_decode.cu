@@ -617,7 +617,7 @@ int sm_count_dec() {
 }
 
 template <int NT, int MB, int KW>
-cudaError_t launch_nt(const DecParams<MB>& P, int grid, cudaStream_t s) {
+cudaError_t launch_nt(const DecParams<MB>& P, int grid, cudaStream_t s, bool overlap) {
   static std::once_flag once;
   static cudaError_t attr_err = cudaSuccess;
   std::call_once(once, []() {
@@ -633,7 +633,7 @@ cudaError_t launch_nt(const DecParams<MB>& P, int grid, cudaStream_t s) {
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = overlap ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, k_decode<NT, MB, KW>, P);
 }
 
@@ -810,6 +810,8 @@ gs_status launch_decode(const gs_packed* const* ps, const void* const* xs, void*
   P.sched = first_slot->cnt + (size_t)ps[0]->nblk64 * kDW;
   P.inject_ns = take_injected_wait(GS_ALGO_DECODE);
   const int grid = (int)std::min<int64_t>(units, max_grid);
+  bool overlap = true;
+  for (int i = 0; i < n; ++i) overlap &= may_overlap(ps[i], s);
   cudaError_t e;
   if (n <= kSmallBatch) {
     DecParams<kSmallBatch> Q;
@@ -820,11 +822,11 @@ gs_status launch_decode(const gs_packed* const* ps, const void* const* xs, void*
     Q.sched = P.sched;
     Q.err = P.err;
     Q.inject_ns = P.inject_ns;
-    if (kw == 256) e = T <= 8 ? launch_nt<1, kSmallBatch, 256>(Q, grid, s) : launch_nt<2, kSmallBatch, 256>(Q, grid, s);
-    else e = T <= 8 ? launch_nt<1, kSmallBatch, 128>(Q, grid, s) : launch_nt<2, kSmallBatch, 128>(Q, grid, s);
+    if (kw == 256) e = T <= 8 ? launch_nt<1, kSmallBatch, 256>(Q, grid, s, overlap) : launch_nt<2, kSmallBatch, 256>(Q, grid, s, overlap);
+    else e = T <= 8 ? launch_nt<1, kSmallBatch, 128>(Q, grid, s, overlap) : launch_nt<2, kSmallBatch, 128>(Q, grid, s, overlap);
   } else {
-    if (kw == 256) e = T <= 8 ? launch_nt<1, kMaxBatch, 256>(P, grid, s) : launch_nt<2, kMaxBatch, 256>(P, grid, s);
-    else e = T <= 8 ? launch_nt<1, kMaxBatch, 128>(P, grid, s) : launch_nt<2, kMaxBatch, 128>(P, grid, s);
+    if (kw == 256) e = T <= 8 ? launch_nt<1, kMaxBatch, 256>(P, grid, s, overlap) : launch_nt<2, kMaxBatch, 256>(P, grid, s, overlap);
+    else e = T <= 8 ? launch_nt<1, kMaxBatch, 128>(P, grid, s, overlap) : launch_nt<2, kMaxBatch, 128>(P, grid, s, overlap);
   }
   note_launch();
   return e == cudaSuccess ? GS_OK : GS_ERR_CUDA;

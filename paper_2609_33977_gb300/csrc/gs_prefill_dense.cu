@@ -1259,7 +1259,9 @@ gs_status launch_prefill_dense(const void* const* xs, const gs_packed* const* ps
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 2;
+    bool overlap = true;
+    for (int k = 0; k < nb; ++k) overlap &= may_overlap(ps[order[b0 + k]], s);
+    cfg.numAttrs = overlap ? 2 : 1;
     bool any_split = false;
     for (int k = 0; k < nb; ++k) any_split |= parts[k] > 1;
     const cudaError_t e = any_split  ? (kw == 128 ? d_launch<128, 0, 256, true>(cfg, P) : d_launch<256, 0, 256, true>(cfg, P))
