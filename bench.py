@@ -553,7 +553,7 @@ def run_ours(args):
         cpu = oracle_sample_rate(w_o, layers_o, args.cpu_seconds)
         cpu["single_thread"] = oracle_single_thread_rate(args.cpu_seconds / 2)
 
-    traffic = recorded_traffic("k_decode", "gs_decode.cu", "llama2-13b-block")
+    traffic = recorded_traffic("k_prefill_dense", "gs_prefill_dense.cu", "llama2-13b-block")
     line = {
         "metric": METRIC, "value": value, "unit": "tokens/s", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": 1e3 * elapsed / args.steps, "higher_is_better": True,
@@ -565,7 +565,7 @@ def run_ours(args):
                    "parallelism": f"replicas x{world}",
                    "graph": f"one CUDA graph per step: {launches_per_step} batched decode launches "
                             f"(one per block per T)"},
-        "roofline": {"kernel": "k_decode", "bound": "hbm", "achieved": achieved_gbs, "peak": hbm_peak, "unit": "GB/s",
+        "roofline": {"kernel": "k_prefill_dense", "bound": "hbm", "achieved": achieved_gbs, "peak": hbm_peak, "unit": "GB/s",
                      "frac": achieved_gbs / hbm_peak, "peak_source": f"{peaks_src} hbm_gbs",
                      "bytes_per_step": bytes_per_step, "launches_per_step": launches_per_step,
                      "algorithmic_bytes_per_launch": bytes_per_step / launches_per_step, "traffic": traffic,
