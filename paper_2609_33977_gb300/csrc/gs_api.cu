@@ -25,7 +25,7 @@ std::atomic<uint64_t> g_inject_ns[4] = {{0}, {0}, {0}, {0}};
 
 // Token count at and above which gs_linear uses the tensor-core kernels: one
 // decode launch covers up to 16 tokens, while the tensor-core kernels' time is
-// nearly flat up to 128.  At T = 17 / 32 a batched LLaMA-2-13B block takes 71 us
+// nearly flat up to 64.  At T = 17 / 32 a batched LLaMA-2-13B block takes 58 us
 // there against 144-156 us as two decode launches (72 us for one at T = 16).
 constexpr int64_t kPrefillMinTokens = 17;
 

@@ -717,8 +717,8 @@ gs_status sq_linear_batched(const void* const* xs, const gs_packed* const* ps, i
     //    flat up to 128 tokens.  For layers whose input is whole 128-column items,
     //    g <= 64, the zero-filled-window kernel is ahead from the second launch on
     //    (us per block at T = 16 / 32, decode against zero-filled: 7B 16x16 52 / 100
-    //    against 67 / 67, 64x64 41 / 81 against 48 / 48, Qwen2.5-7B 32x32 52 / 103
-    //    against 86 / 86); the square tensor-core kernel
+    //    against 67 / 67, 64x64 41 / 81 against 40 / 40, Qwen2.5-7B 32x32 52 / 103
+    //    against 64 / 64); the square tensor-core kernel
     //    (the other layers) breaks even at 128 / 64 / 32 / 16 tokens for
     //    g = 16 / 32 / 64 / 128;
     //  - above it, the zero-filled-window kernel where it applies (dense-layer

@@ -10,8 +10,8 @@
 // register full of zeros:
 //   packed tiles --TMA box--> shared (the half window's kept rows, compact)
 //     --ld.shared by kept lanes--> registers --tcgen05.st--> TMEM A slot.
-// x is the B operand (TMA, 128-byte swizzle).  Per 128-deep K stage the leader
-// issues eight M = 256 x N x 16 cta_group::2 MMAs; D^T (rows x tokens, fp32)
+// x is the B operand (TMA, 128-byte swizzle).  Per K stage (128 deep, or 256 at N <= 128)
+// the leader issues M = 256 x N x 16 cta_group::2 MMAs; D^T (rows x tokens, fp32)
 // stays in TMEM for the whole unit.
 //
 // Why this split.  Shared memory receives x (N / 2 x 256 B a stage) and the kept
@@ -21,12 +21,13 @@
 // fences and the second operand's bytes held a 7B block at T = 2048 to 547 us,
 // 1.52 PFLOP/s dense-equivalent; now 405 us, 2.05 PFLOP/s, at the chip's power limit.)
 //
-// What bounds it.  At N = 256 the tensor cores.  At small N the chain of hand-offs
-// of a stage (copy -> converters -> leader -> commit), about 0.45 us a stage of 128
-// k: 13B block at T = 32 / 128 in 71 / 76 us (4.5 TB/s of kept weights at T = 32).
-// The roles that issue MMAs and copies walk their stages with the whole warp and
-// issue from one elected lane: inside a one-lane branch an MMA cost 70 cycles of
-// issue and a copy 220 to 400 (13B block at T = 128: 92 us).
+// What bounds it.  At N = 256 the tensor cores.  At small N the stream of kept weights
+// (5.7 TB/s) and, where units are few, the chain of hand-offs of a stage (copy ->
+// converters -> leader -> commit), about 0.35 us however deep the stage is: 13B block at
+// T = 32 / 128 in 58 / 67 us with 256-deep stages, 71 / 76 us with 128.  The roles that
+// issue MMAs and copies walk their stages with the whole warp and issue from one elected
+// lane: inside a one-lane branch an MMA cost 70 cycles of issue and a copy 220 to 400
+// (13B block at T = 128, 128-deep: 92 us).
 //
 // Roles (one CTA per SM, units persistent over the pairs): warp 0 x copies,
 // warp 1 W copies, warp 2 TMEM allocator + MMA issuer (leader), warps 4..11
@@ -85,8 +86,8 @@ constexpr bool d_ring_holds_two(int sk, int n_max) {
   return true;
 }
 static_assert(d_ring_holds_two(128, kDN) && d_ring_holds_two(256, kDN / 2), "two largest W stages fit the ring");
-// TMEM columns of D (n <= 64: two buffers), and the A slots the rest holds: a slot's
-// round trip (both CTAs' converters, the leader, the commit) is about 1.4 us
+// TMEM columns of D (n <= 64: two buffers), and the A slots the rest holds: six
+// 128-deep slots at n <= 128 measured no faster than four
 __host__ __device__ constexpr uint32_t d_d_cols(int n) { return n <= kDN / 2 ? kDN / 2 : kDN; }
 __host__ __device__ constexpr uint32_t d_a_slots(int n, int sk) { return (512 - d_d_cols(n)) / (uint32_t)(sk / 2); }
 static_assert(d_a_slots(kDN, 128) == 4 && d_a_slots(kDN / 2, 256) == 3, "A slots no more than x slots");
@@ -224,8 +225,7 @@ __device__ __forceinline__ bool d_wait_warp(uint64_t* bar, uint32_t parity, vola
 
 // Walks a pair's units in batches of 32 items.  Lane l of a warp looks after
 // item c0 + l of the batch; what it loads for the next batch is in flight while
-// the warp works through this one.  (Loaded an item ahead instead, the lookups
-// queue behind the copies in flight: 1.0 us a stage instead of 0.5.)
+// the warp works through this one.
 template <int SQ, int kCh, bool kSplit>
 struct DWalk {
   const DParams* P;
@@ -1110,8 +1110,7 @@ int64_t d_token_tiles(const std::vector<int64_t>& units, const std::vector<int64
 
 // Which 1 x KW layers take this kernel: all that have kept groups, in the whole
 // prefill regime.  Against the gathering kernel, d = 0.5, us per batched block:
-// 13B 1 x 256 at T = 17 / 128 / 256 / 512 71 / 76 / 93 / 168 against 92 / 98 / 173 / 294;
-// 7B 1 x 128 at T = 32 / 128 50 / 54 against 78 / 101.  One call per layer, over
+// 13B 1 x 256 at T = 32 / 128 / 512 58 / 67 / 168 against 93 / 98 / 294.  One call per layer, over
 // nine shapes from 1024 x 1024 to 20000 x 1024 and T = 17 to 640, it takes
 // 0.4-0.97x the gathering kernel's time.
 bool prefill_prefers_dense(const gs_packed* p, int64_t T) {
