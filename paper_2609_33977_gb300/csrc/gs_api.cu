@@ -354,11 +354,11 @@ static gs_status linear_impl(const void* x_dev, const gs_packed* p, int64_t T, v
   if (algo == GS_ALGO_AUTO) {
     // the same per-layer choice as gs_linear_batched makes
     if (T < kPrefillMinTokens) {
-      if (prefill_prefers_dense(p, T) && decode_prefers_dense(&p, 1, T))
+      if (prefill_prefers_dense(p) && decode_prefers_dense(&p, 1, T))
         return launch_prefill_dense(&x_dev, &p, 1, T, &y_dev, s, nullptr, true);
       algo = GS_ALGO_DECODE;
     }
-    else if (prefill_prefers_dense(p, T)) algo = GS_ALGO_PREFILL_DENSE;
+    else if (prefill_prefers_dense(p)) algo = GS_ALGO_PREFILL_DENSE;
     else algo = p->G <= prefill_max_chunks() ? GS_ALGO_PREFILL : GS_ALGO_DECODE;
   }
   if (algo == GS_ALGO_PREFILL) return launch_prefill(x_dev, p, T, y_dev, s);
@@ -451,7 +451,7 @@ gs_status gs_linear_batched(int32_t n, const void* const* xs_dev, const gs_packe
     std::vector<const gs_packed*> pp, pd;
     std::vector<void*> yp, yd;
     for (int i = 0; i < n; ++i) {
-      if (prefill_prefers_dense(ps[i], T)) {
+      if (prefill_prefers_dense(ps[i])) {
         xd.push_back(xs_dev[i]);
         pd.push_back(ps[i]);
         yd.push_back(ys_dev[i]);
@@ -474,7 +474,7 @@ gs_status gs_linear_batched(int32_t n, const void* const* xs_dev, const gs_packe
   if (decode_prefers_dense(ps, n, T)) {
     std::vector<int> idx;
     for (int i = 0; i < n; ++i) {
-      if (prefill_prefers_dense(ps[i], T)) idx.push_back(i);
+      if (prefill_prefers_dense(ps[i])) idx.push_back(i);
       else if (cudaMemsetAsync(ys_dev[i], 0, (size_t)T * (size_t)ps[i]->out * 2, s) != cudaSuccess) return GS_ERR_CUDA;
     }
     return launch_prefill_dense(xs_dev, ps, (int)idx.size(), T, ys_dev, s, idx.data(), true);

@@ -190,8 +190,8 @@ int prefill_max_chunks();
 // split along the input, with the decode path's per-stream scratch (1 x KW layers).
 gs_status launch_prefill_dense(const void* const* xs, const gs_packed* const* ps, int n, int64_t T, void* const* ys,
                                cudaStream_t s, const int* idx = nullptr, bool split = false);
-// whether the zero-filled kernel is the faster one for this layer and token count
-bool prefill_prefers_dense(const gs_packed* p, int64_t T);
+// whether the zero-filled kernel takes this layer in the prefill regime
+bool prefill_prefers_dense(const gs_packed* p);
 // whether a call of at most 16 tokens over these 1 x KW layers (one chunk width) takes it, split
 bool decode_prefers_dense(const gs_packed* const* ps, int n, int64_t T);
 

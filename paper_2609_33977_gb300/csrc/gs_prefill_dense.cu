@@ -61,6 +61,7 @@ constexpr int kDThreads = (kDEpiWarp0 + kDEpiWarps) * 32;
 constexpr int kDMmaWarp = 2;
 constexpr uint32_t kDTmemCols = 512;              // D first, then the A slots of 64 columns each
 constexpr int kDMaxLayers = 8;
+constexpr int kDMaxChunks = 32767;                // wider inputs stay on the other kernels
 constexpr int kDWMaps = 8;                        // W box heights: 16, 32, ..., 128 rows (square: g, 2g, ..., 128)
 constexpr uint64_t kDWaitLimitNs = 2000000000ull;
 constexpr uint64_t kDDrainLimitNs = 200000000ull;
@@ -1113,9 +1114,8 @@ int64_t d_token_tiles(const std::vector<int64_t>& units, const std::vector<int64
 // 13B 1 x 256 at T = 32 / 128 / 512 58 / 67 / 168 against 93 / 98 / 294.  One call per layer, over
 // nine shapes from 1024 x 1024 to 20000 x 1024 and T = 17 to 640, it takes
 // 0.4-0.97x the gathering kernel's time.
-bool prefill_prefers_dense(const gs_packed* p, int64_t T) {
-  (void)T;
-  return p->kept > 0 && p->g_out == 1 && (p->g_in == 128 || p->g_in == 256);
+bool prefill_prefers_dense(const gs_packed* p) {
+  return p->kept > 0 && p->g_out == 1 && (p->g_in == 128 || p->g_in == 256) && p->G <= kDMaxChunks;
 }
 
 // Whether a call of at most 16 tokens over layers of one chunk width takes this
@@ -1131,7 +1131,10 @@ bool prefill_prefers_dense(const gs_packed* p, int64_t T) {
 bool decode_prefers_dense(const gs_packed* const* ps, int n, int64_t T) {
   if (T > 16) return false;
   int64_t weights = 0;
-  for (int i = 0; i < n; ++i) weights += ps[i]->out * ps[i]->in;
+  for (int i = 0; i < n; ++i) {
+    if (ps[i]->kept > 0 && !prefill_prefers_dense(ps[i])) return false;
+    weights += ps[i]->out * ps[i]->in;
+  }
   if (T <= 2 && n > 1 && ps[0]->g_in == 256) return weights >= 250000000;
   return weights >= 20000000;
 }
@@ -1214,7 +1217,7 @@ gs_status launch_prefill_dense(const void* const* xs, const gs_packed* const* ps
         L.nw = p->nw16;
         L.G = p->G;
       }
-      if (L.G > 32767) return GS_ERR_UNSUPPORTED;
+      if (L.G > kDMaxChunks) return GS_ERR_UNSUPPORTED;
       L.n_m = (int32_t)n_m;
       L.tile_begin = (int32_t)tiles;
       tiles += (int64_t)L.n_m * L.n_split * ((p->out + kDW - 1) / kDW);
