@@ -125,20 +125,26 @@ void handles_used(const gs_packed* const* ps, int n, cudaStream_t s) {
   }
 }
 
-bool may_overlap(const gs_packed* p, cudaStream_t s) {
-  // any other stream is ordered after packing by an event, a full dependency (the
-  // legacy stream has two names)
+// s is gs_pack's stream (the legacy stream has two names)
+static bool on_pack_stream(const gs_packed* p, cudaStream_t s) {
   const auto one_name = [](void* x) { return x == static_cast<void*>(cudaStreamLegacy) ? nullptr : x; };
-  if (one_name(static_cast<void*>(s)) != one_name(p->pack_stream)) return true;
+  return one_name(static_cast<void*>(s)) == one_name(p->pack_stream);
+}
+
+bool may_overlap(const gs_packed* p, cudaStream_t s) {
+  // any other stream is ordered after packing by an event, a full dependency
+  return !__atomic_load_n(&p->fresh, __ATOMIC_ACQUIRE) || !on_pack_stream(p, s);
+}
+
+void launch_queued(const gs_packed* p, cudaStream_t s) {
   int32_t* fresh = const_cast<int32_t*>(&p->fresh);
-  if (!__atomic_load_n(fresh, __ATOMIC_ACQUIRE)) return true;
-  if (s == cudaStreamPerThread) return false;   // another stream in every thread
+  if (!__atomic_load_n(fresh, __ATOMIC_RELAXED) || !on_pack_stream(p, s)) return;
+  if (s == cudaStreamPerThread) return;   // another stream in every thread
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
   const cudaError_t e = cudaStreamIsCapturing(s, &st);
   if (e != cudaSuccess) cudaGetLastError();
   // a captured launch does not run now: the next one on the stream may still follow packing
   if (e == cudaSuccess && st == cudaStreamCaptureStatusNone) __atomic_store_n(fresh, 0, __ATOMIC_RELEASE);
-  return false;
 }
 
 void handle_on_stream(gs_packed* p, cudaStream_t s) {

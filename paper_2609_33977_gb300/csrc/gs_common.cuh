@@ -54,7 +54,7 @@ struct gs_packed {
   int32_t nbufs;
   gs::PoolTag tag;
   void* pack_stream;   // cudaStream_t, compared only
-  int32_t fresh;       // atomic: no launch has followed packing on its stream yet (see may_overlap)
+  int32_t fresh;       // atomic: no launch has been queued behind packing on its stream yet (see may_overlap)
   int32_t shared;      // atomic: used on another stream than gs_pack's, or captured into a graph
   int64_t out, in;
   int32_t G;          // in / 256
@@ -134,9 +134,12 @@ void handle_on_stream(gs_packed* p, cudaStream_t s);
 void handles_used(const gs_packed* const* ps, int n, cudaStream_t s);
 // Whether a launch on s may use programmatic dependent launch.  The decode and
 // zero-filled kernels read weights and their index before they wait for the launch
-// before them, which is only sound while that launch is not the packing itself: a
-// handle's first launch on its pack stream is an ordinary one.
+// before them, which is only sound while that launch is not the packing itself: until
+// an ordinary launch of a handle is in its pack stream (launch_queued), every launch of
+// it there is an ordinary one, whichever thread asks.
 bool may_overlap(const gs_packed* p, cudaStream_t s);
+// a launch over p that may not overlap has been queued on s, without error
+void launch_queued(const gs_packed* p, cudaStream_t s);
 // waits for s and reads the kept-group count into p->kept
 gs_status read_kept(gs_packed* p, const int64_t* kept_dev, cudaStream_t s);
 // pool.cu: idle device buffers of released handles

@@ -829,7 +829,10 @@ gs_status launch_decode(const gs_packed* const* ps, const void* const* xs, void*
     else e = T <= 8 ? launch_nt<1, kMaxBatch, 128>(P, grid, s, overlap) : launch_nt<2, kMaxBatch, 128>(P, grid, s, overlap);
   }
   note_launch();
-  return e == cudaSuccess ? GS_OK : GS_ERR_CUDA;
+  if (e != cudaSuccess) return GS_ERR_CUDA;
+  if (!overlap)
+    for (int i = 0; i < n; ++i) launch_queued(ps[i], s);
+  return GS_OK;
 }
 
 }  // namespace gs

@@ -1274,6 +1274,8 @@ gs_status launch_prefill_dense(const void* const* xs, const gs_packed* const* ps
                                       : (deep ? d_launch<256, 0, 256>(cfg, P) : d_launch<256, 0, 128>(cfg, P));
     note_launch();
     if (e != cudaSuccess) return GS_ERR_CUDA;
+    if (!overlap)
+      for (int k = 0; k < nb; ++k) launch_queued(ps[order[b0 + k]], s);
   }
   return GS_OK;
 }
