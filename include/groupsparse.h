@@ -255,11 +255,20 @@ gs_status gs_pack_index_noalloc(const uint8_t* mask_dev, int64_t out, int64_t in
  * completes.  If the handle was used on gs_pack's stream only, and not inside a
  * graph capture, its device buffers are kept for the next gs_pack on that
  * stream, at most 1/128 of the device's memory in all; they return to the
- * device when that is exceeded, when they stay unused, or when an allocation of
- * the library finds the device out of memory.  Otherwise they are freed at
- * once (cudaFree, which waits for the device).
+ * device when that is exceeded, when 8192 other buffers (about 450 packed and
+ * released handles) have come and gone since, when an allocation of the library
+ * finds the device out of memory, or with gs_trim.  A program that stops
+ * packing and releasing keeps them until then: other allocators do not see
+ * them.  Buffers of any other handle are freed at once (cudaFree, which waits
+ * for the device).
  */
 void gs_free(gs_packed* p);
+
+/*
+ * Gives the device buffers that gs_free kept back to the device, of every
+ * stream (cudaFree, which waits for the device: not while a stream captures).
+ */
+void gs_trim(void);
 
 /* Static description of a status code. */
 const char* gs_status_string(gs_status s);

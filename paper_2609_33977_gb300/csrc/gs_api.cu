@@ -65,7 +65,7 @@ int* device_error_flag() {
   std::lock_guard<std::mutex> lk(g_flag_mu);
   if (!g_flags[dev]) {
     int* f = nullptr;
-    if (cudaMalloc(&f, 2 * sizeof(int)) != cudaSuccess) return nullptr;
+    if (device_malloc(reinterpret_cast<void**>(&f), 2 * sizeof(int)) != cudaSuccess) return nullptr;
     if (cudaMemset(f, 0, 2 * sizeof(int)) != cudaSuccess) {
       cudaFree(f);
       return nullptr;
@@ -199,17 +199,12 @@ gs_status read_kept(gs_packed* p, const int64_t* kept_dev, cudaStream_t s) {
 gs_status lib_malloc(void** ptr, size_t bytes) {
   *ptr = nullptr;
   if (fail_this_alloc()) return GS_ERR_OOM;
-  const cudaError_t e = cudaMalloc(ptr, bytes);
+  const cudaError_t e = device_malloc(ptr, bytes);
   if (e == cudaErrorMemoryAllocation) {
     cudaGetLastError();
-    *ptr = nullptr;
     return GS_ERR_OOM;
   }
-  if (e != cudaSuccess) {
-    *ptr = nullptr;
-    return GS_ERR_CUDA;
-  }
-  return GS_OK;
+  return e == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
 
 uint64_t take_injected_wait(int family) {
@@ -555,6 +550,8 @@ void gs_free(gs_packed* p) {
   free_buffers(p);
   delete p;
 }
+
+void gs_trim(void) { pool_trim(); }
 
 const char* gs_status_string(gs_status s) {
   switch (s) {

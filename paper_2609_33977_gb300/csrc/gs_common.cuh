@@ -121,11 +121,12 @@ void note_launch(int64_t n = 1);
 // Incremented each time gs_device_status reports a timeout: scratch whose
 // arrival counters were last cleaned at an older epoch is re-zeroed first.
 uint64_t timeout_epoch();
-// Every device allocation of the library goes through here (so that a test can
-// make the n-th one fail); OOM on cudaErrorMemoryAllocation, else CUDA.
+// Device allocations of the library, so that a test can make the n-th one fail (the
+// error flags excepted); OOM on cudaErrorMemoryAllocation, else CUDA.  lib_malloc is
+// for the split scratch of streams other than a handle's pack stream.
 gs_status lib_malloc(void** ptr, size_t bytes);
-// the same for a buffer that handle p owns: it comes from the pool and returns
-// there, or to cudaFree, with the handle
+// for a buffer that handle p owns: it comes from the pool and returns there, or to
+// cudaFree, with the handle
 gs_status handle_malloc(gs_packed* p, void** ptr, size_t bytes);
 void handle_free(gs_packed* p, const void* ptr);   // one of them, before the handle goes
 // fills in the pack stream and its identity
@@ -146,6 +147,9 @@ gs_status read_kept(gs_packed* p, const int64_t* kept_dev, cudaStream_t s);
 PoolTag pool_tag(int device, cudaStream_t s);
 cudaError_t pool_take(PoolBuf* buf, size_t bytes, const PoolTag& tag);
 void pool_give(const PoolBuf& buf, const PoolTag& tag);   // an invalid tag: cudaFree
+void pool_trim();                                         // cudaFree of every idle buffer
+// cudaMalloc that gives the idle buffers back and tries again when the device is full
+cudaError_t device_malloc(void** ptr, size_t bytes);
 // Test hook: limit of a wait on the never-set word to inject into the next
 // launch of a kernel family (GS_ALGO_DECODE / GS_ALGO_PREFILL /
 // GS_ALGO_PREFILL_DENSE); 0 = none.

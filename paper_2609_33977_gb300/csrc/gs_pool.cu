@@ -16,8 +16,10 @@
 // the device.
 //
 // What is kept is bounded (1 / 128 of the device's memory, oldest released
-// first), is released when it has not been used for a while (kPoolMaxAge
-// releases of other buffers) and when the device is out of memory.
+// first).  It goes back to the device when kPoolMaxAge other buffers have been
+// taken or released since, when any allocation of the library finds the device
+// full, and when the caller asks (gs_trim).  A program that neither packs nor
+// releases handles any more keeps it until then.
 #include "gs_common.cuh"
 
 #include <mutex>
@@ -28,17 +30,17 @@ namespace {
 struct Idle {
   PoolBuf buf;
   PoolTag tag;
-  uint64_t since;   // tick of its release
+  uint64_t since;   // g_tick at its release
 };
 
 constexpr int kMaxIdle = 256;
-constexpr uint64_t kPoolMaxAge = 4096;
+constexpr uint64_t kPoolMaxAge = 8192;   // a handle takes and releases about nine
 
 std::mutex g_pool_mu;
 Idle g_idle[kMaxIdle];   // oldest first
 int g_n_idle = 0;
 size_t g_idle_bytes = 0;
-uint64_t g_tick = 0;
+uint64_t g_tick = 0;     // buffers taken and released so far
 
 size_t idle_limit() {
   static const size_t limit = []() {
@@ -95,7 +97,29 @@ bool release_oldest(F which) {
   return true;
 }
 
+void release_aged() {
+  while (release_oldest([]() { return g_tick - g_idle[0].since > kPoolMaxAge; })) {
+  }
+}
+
 }  // namespace
+
+void pool_trim() {
+  while (release_oldest([]() { return true; })) {
+  }
+}
+
+cudaError_t device_malloc(void** ptr, size_t bytes) {
+  *ptr = nullptr;
+  cudaError_t e = cudaMalloc(ptr, bytes);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    pool_trim();
+    e = cudaMalloc(ptr, bytes);
+  }
+  if (e != cudaSuccess) *ptr = nullptr;
+  return e;
+}
 
 PoolTag pool_tag(int device, cudaStream_t s) {
   PoolTag t{device, false, 0};
@@ -114,6 +138,7 @@ cudaError_t pool_take(PoolBuf* buf, size_t bytes, const PoolTag& tag) {
   const size_t want = round_size(bytes);
   {
     std::lock_guard<std::mutex> lk(g_pool_mu);
+    ++g_tick;
     int best = -1;
     for (int i = 0; i < g_n_idle; ++i)
       if (same(g_idle[i].tag, tag) && g_idle[i].buf.bytes >= want && g_idle[i].buf.bytes - want <= want / 8 &&
@@ -125,14 +150,9 @@ cudaError_t pool_take(PoolBuf* buf, size_t bytes, const PoolTag& tag) {
       return cudaSuccess;
     }
   }
+  release_aged();
   void* ptr = nullptr;
-  cudaError_t e = cudaMalloc(&ptr, want);
-  if (e == cudaErrorMemoryAllocation) {
-    cudaGetLastError();
-    while (release_oldest([]() { return true; })) {
-    }
-    e = cudaMalloc(&ptr, want);
-  }
+  const cudaError_t e = device_malloc(&ptr, want);
   if (e == cudaSuccess) *buf = PoolBuf{ptr, want};
   return e;
 }
@@ -152,8 +172,7 @@ void pool_give(const PoolBuf& buf, const PoolTag& tag) {
     }
   }
   if (!kept) free_on(tag.device, buf.ptr);
-  while (release_oldest([]() { return g_tick - g_idle[0].since > kPoolMaxAge; })) {
-  }
+  release_aged();
 }
 
 }  // namespace gs

@@ -42,6 +42,8 @@ def _load(path: Path = LIB_PATH) -> ctypes.CDLL:
     lib.gs_packed_export.argtypes = [vp, _c_i64p, _c_i32p, _c_u16p, _c_i32p, _c_u16p]
     lib.gs_free.argtypes = [vp]
     lib.gs_free.restype = None
+    lib.gs_trim.argtypes = []
+    lib.gs_trim.restype = None
     lib.gs_status_string.argtypes = [ctypes.c_int]
     lib.gs_status_string.restype = ctypes.c_char_p
     lib.gs_device_status.argtypes = [vp]
@@ -154,6 +156,11 @@ class Packed:
             self.free()
         except Exception:
             pass
+
+
+def trim() -> None:
+    """Give the device buffers kept from released handles back to the device (waits for it)."""
+    lib.gs_trim()
 
 
 def pack(W: torch.Tensor, mask: torch.Tensor, stream: Optional[torch.cuda.Stream] = None) -> Packed:

@@ -50,6 +50,8 @@ cudaError_t cudaStreamGetId(cudaStream_t s, unsigned long long* id) { *id = (uns
 cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* st) { ++g_asked; *st = g_capture; return cudaSuccess; }
 }
 
+void gs::decode_release(gs_packed*) {}   // no scratch of other streams here
+
 #define CHECK(c) do { if (!(c)) { std::printf("line %d: %s\n", __LINE__, #c); std::exit(1); } } while (0)
 static cudaStream_t stream(int i) { return reinterpret_cast<cudaStream_t>((uintptr_t)(i * 64)); }   // 0: the legacy stream
 // a handle as gs_pack leaves it
@@ -108,4 +110,64 @@ def test_no_launch_overlaps_packing_until_an_ordinary_one_is_queued(run, s):
       CHECK(!gs::may_overlap(r, cudaStreamLegacy));
       gs::launch_queued(r, cudaStreamLegacy);
       CHECK(gs::may_overlap(r, stream(0)));
+    """)
+
+
+def test_any_allocation_that_finds_the_device_full_releases_idle_buffers(run):
+    """The split scratch of a second stream (lib_malloc) as well as a handle's own buffers."""
+    run("full", """
+      g_capacity = 100 << 20;
+      gs_packed* p = packed(stream(1));
+      void *a = nullptr, *b = nullptr;
+      CHECK(gs::handle_malloc(p, &a, 60 << 20) == GS_OK);
+      gs_free(p);
+      CHECK(g_used == (60 << 20));                          // kept, idle
+      CHECK(gs::lib_malloc(&b, 90 << 20) == GS_OK && b);    // fits only once it is gone
+      CHECK(g_used == (90 << 20));
+      CHECK(gs::lib_malloc(&a, 90 << 20) == GS_ERR_OOM && !a);
+      cudaFree(b);
+      p = packed(stream(1));
+      CHECK(gs::handle_malloc(p, &a, 60 << 20) == GS_OK);
+      gs_free(p);
+      gs_packed* q = packed(stream(2));
+      CHECK(gs::handle_malloc(q, &a, 90 << 20) == GS_OK);
+      gs_free(q);
+    """)
+
+
+def test_idle_buffers_age_in_packs_and_releases(run):
+    """A program that goes on packing without releasing gives unused buffers back too."""
+    run("age", """
+      gs_packed* p = packed(stream(1));
+      void* a = nullptr;
+      CHECK(gs::handle_malloc(p, &a, 1 << 20) == GS_OK);
+      gs_free(p);
+      CHECK(g_live.size() == 1);
+      gs_packed* q = packed(stream(2));                 // other stream: does not take it
+      CHECK(gs::handle_malloc(q, &a, 512) == GS_OK);
+      CHECK(g_live.size() == 2);
+      for (int i = 0; i < 1000; ++i) {
+        gs_packed* r = packed(stream(2));
+        for (int k = 0; k < 9; ++k) CHECK(gs::handle_malloc(r, &a, 512) == GS_OK);   // never released
+      }
+      CHECK(g_live.size() == 1 + 9000);
+    """)
+
+
+def test_trim_gives_every_idle_buffer_back_and_keeps_those_in_use(run):
+    run("trim", """
+      void* a = nullptr;
+      gs_packed* keep = packed(stream(1));
+      CHECK(gs::handle_malloc(keep, &a, 4096) == GS_OK);
+      for (int s = 0; s < 3; ++s) {
+        gs_packed* p = packed(stream(s));
+        for (int k = 0; k < 5; ++k) CHECK(gs::handle_malloc(p, &a, (size_t)1 << (10 + k)) == GS_OK);
+        gs_free(p);
+      }
+      CHECK(g_live.size() == 16);
+      gs_trim();
+      CHECK(g_live.size() == 1 && g_used == 4096);
+      gs_free(keep);
+      gs_trim();
+      CHECK(g_live.empty());
     """)
