@@ -62,6 +62,8 @@ gs_status check_handle(const gs_packed* p) {
 int* device_error_flag() {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+  int* made = __atomic_load_n(&g_flags[dev], __ATOMIC_ACQUIRE);
+  if (made) return made;
   std::lock_guard<std::mutex> lk(g_flag_mu);
   if (!g_flags[dev]) {
     int* f = nullptr;
@@ -70,7 +72,7 @@ int* device_error_flag() {
       cudaFree(f);
       return nullptr;
     }
-    g_flags[dev] = f;
+    __atomic_store_n(&g_flags[dev], f, __ATOMIC_RELEASE);
   }
   return g_flags[dev];
 }
@@ -110,18 +112,27 @@ void handle_free(gs_packed* p, const void* ptr) {
   }
 }
 
+// Work queued on s goes into a graph.  The legacy stream cannot be captured, so the
+// driver is not asked there.
+static bool captured(cudaStream_t s) {
+  if (s == nullptr || s == cudaStreamLegacy) return false;
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  const cudaError_t e = cudaStreamIsCapturing(s, &st);
+  if (e != cudaSuccess) cudaGetLastError();   // the launch reports what is wrong with s
+  return e != cudaSuccess || st != cudaStreamCaptureStatusNone;
+}
+
 void handles_used(const gs_packed* const* ps, int n, cudaStream_t s) {
-  int captured = -1;   // asked at most once per call
+  int in_graph = -1;   // asked at most once per call
   for (int i = 0; i < n; ++i) {
-    int32_t* shared = const_cast<int32_t*>(&ps[i]->shared);   // the one mutable field besides the scratch table
+    int32_t* shared = const_cast<int32_t*>(&ps[i]->shared);   // mutable, as the scratch table is
     if (__atomic_load_n(shared, __ATOMIC_RELAXED)) continue;
-    if (captured < 0) {
-      cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-      const cudaError_t e = cudaStreamIsCapturing(s, &st);
-      if (e != cudaSuccess) cudaGetLastError();   // the launch that follows reports what is wrong with s
-      captured = e != cudaSuccess || st != cudaStreamCaptureStatusNone ? 1 : 0;
+    bool leaves = static_cast<void*>(s) != ps[i]->pack_stream;
+    if (!leaves) {
+      if (in_graph < 0) in_graph = captured(s) ? 1 : 0;
+      leaves = in_graph != 0;
     }
-    if (captured || static_cast<void*>(s) != ps[i]->pack_stream) __atomic_store_n(shared, 1, __ATOMIC_RELEASE);
+    if (leaves) __atomic_store_n(shared, 1, __ATOMIC_RELEASE);
   }
 }
 
@@ -140,11 +151,8 @@ void launch_queued(const gs_packed* p, cudaStream_t s) {
   int32_t* fresh = const_cast<int32_t*>(&p->fresh);
   if (!__atomic_load_n(fresh, __ATOMIC_RELAXED) || !on_pack_stream(p, s)) return;
   if (s == cudaStreamPerThread) return;   // another stream in every thread
-  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  const cudaError_t e = cudaStreamIsCapturing(s, &st);
-  if (e != cudaSuccess) cudaGetLastError();
   // a captured launch does not run now: the next one on the stream may still follow packing
-  if (e == cudaSuccess && st == cudaStreamCaptureStatusNone) __atomic_store_n(fresh, 0, __ATOMIC_RELEASE);
+  if (!captured(s)) __atomic_store_n(fresh, 0, __ATOMIC_RELEASE);
 }
 
 void handle_on_stream(gs_packed* p, cudaStream_t s) {

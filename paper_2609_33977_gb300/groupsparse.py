@@ -79,8 +79,10 @@ def _check(status: int, what: str) -> None:
 
 
 def _stream_ptr(stream: Optional[torch.cuda.Stream] = None) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return int(s.cuda_stream)
+    if stream is not None:
+        return int(stream.cuda_stream)
+    # the current device's current stream, without a Stream object around it
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _require_cuda(t: torch.Tensor, dtype: torch.dtype, name: str) -> None:
@@ -200,7 +202,7 @@ def linear_into(x: torch.Tensor, p: Packed, y: torch.Tensor, algo: int = ALGO_AU
     _require_cuda(x, torch.bfloat16, "x")
     _require_cuda(y, torch.bfloat16, "y")
     T = x.shape[0]
-    if x.dim() != 2 or x.shape[1] != p.inp or tuple(y.shape) != (T, p.out):
+    if x.dim() != 2 or x.shape[1] != p.inp or y.shape != (T, p.out):
         raise ValueError("x must be [T, in] and y [T, out]")
     _check(lib.gs_linear_ex(x.data_ptr(), p.handle, T, y.data_ptr(), _stream_ptr(stream), algo), "gs_linear")
     return y
@@ -223,7 +225,7 @@ def linear_batched_into(xs: Sequence[torch.Tensor], ps: Sequence[Packed], ys: Se
     for x, p, y in zip(xs, ps, ys):
         _require_cuda(x, torch.bfloat16, "x")
         _require_cuda(y, torch.bfloat16, "y")
-        if x.shape[0] != T or x.shape[1] != p.inp or tuple(y.shape) != (T, p.out):
+        if x.shape[0] != T or x.shape[1] != p.inp or y.shape != (T, p.out):
             raise ValueError("every x must be [T, in_i] and y [T, out_i] with one T")
     arr = ctypes.c_void_p * n
     xa = arr(*[x.data_ptr() for x in xs])

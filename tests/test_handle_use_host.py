@@ -171,3 +171,27 @@ def test_trim_gives_every_idle_buffer_back_and_keeps_those_in_use(run):
       gs_trim();
       CHECK(g_live.empty());
     """)
+
+
+def test_capture_is_asked_about_only_where_it_can_be(run):
+    """The legacy stream cannot be captured: a call there asks the driver nothing.  Elsewhere a call
+    asks once, and a handle captured or used on another stream loses its claim to the pool."""
+    run("capture", """
+      gs_packed* p[3] = {packed(stream(0)), packed(stream(0)), packed(stream(0))};
+      g_capture = cudaStreamCaptureStatusActive;   // were it asked
+      for (int i = 0; i < 4; ++i) gs::handles_used(p, 3, stream(0));
+      gs::launch_queued(p[0], stream(0));
+      gs::handles_used(p, 1, stream(0));
+      CHECK(g_asked == 0 && !p[0]->shared && !p[2]->shared && gs::may_overlap(p[0], stream(0)));
+      g_capture = cudaStreamCaptureStatusNone;
+      gs::handles_used(p, 1, stream(1));
+      CHECK(g_asked == 0 && p[0]->shared && !p[1]->shared);
+      gs_packed* q[3] = {packed(stream(1)), packed(stream(1)), packed(stream(2))};
+      gs::handles_used(q, 2, stream(1));
+      CHECK(g_asked == 1 && !q[0]->shared && !q[1]->shared);
+      g_capture = cudaStreamCaptureStatusActive;
+      gs::handles_used(q, 3, stream(1));
+      CHECK(g_asked == 2 && q[0]->shared && q[1]->shared && q[2]->shared);
+      gs::handles_used(q, 3, stream(1));
+      CHECK(g_asked == 2);
+    """)
