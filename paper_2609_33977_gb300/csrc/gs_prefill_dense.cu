@@ -1119,24 +1119,18 @@ bool prefill_prefers_dense(const gs_packed* p) {
 }
 
 // Whether a call of at most 16 tokens over layers of one chunk width takes this
-// kernel (split) rather than the decode kernel: from 20 M weights in all.  Below,
-// the few parts of a window cost more than the decode kernel's finer units (graph
-// replays, us at T = 1 / 16, this kernel against decode: 1024 x 1024 6 / 10 against
-// 5 / 8, 4096 x 4096 10 / 13 against 8 / 11; above: 5120 x 5120 11 / 13 against
-// 12 / 20, 20000 x 1024 9 / 9 against 16 / 31, 7B block 37 / 38 against 38 / 47 and
-// with 1 x 128 groups 40 / 40 against 60 / 65, 13B block 54 / 55 against 56 / 67).
-// At one or two tokens the decode kernel streams a batch of 1 x 256 layers as fast up to
-// about 250 M weights (7B block 40.5 us a call against 39.5, Qwen2.5-7B 44 / 43 as graph
-// replays; 13B block 61 against 56) and its launch is prepared 5 us sooner on the host.
+// kernel (split) rather than the decode kernel.
 bool decode_prefers_dense(const gs_packed* const* ps, int n, int64_t T) {
   if (T > 16) return false;
-  int64_t weights = 0;
+  std::vector<FewTokenLayer> layers;
+  layers.reserve((size_t)n);
   for (int i = 0; i < n; ++i) {
-    if (ps[i]->kept > 0 && !prefill_prefers_dense(ps[i])) return false;
-    weights += ps[i]->out * ps[i]->in;
+    const gs_packed* p = ps[i];
+    if (p->kept == 0) continue;
+    if (!prefill_prefers_dense(p)) return false;
+    layers.push_back({p->out, p->in, 2.0 * (double)p->kept * p->g_in, p->G, p->dec_cpu, p->dec_cpu_fine});
   }
-  if (T <= 2 && n > 1 && ps[0]->g_in == 256) return weights >= 250000000;
-  return weights >= 20000000;
+  return !layers.empty() && zero_filled_first(layers, ps[0]->g_in, (int)T, d_sm_count());
 }
 
 gs_status launch_prefill_dense(const void* const* xs, const gs_packed* const* ps, int n, int64_t T, void* const* ys,
