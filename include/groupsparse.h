@@ -53,7 +53,8 @@ typedef enum gs_algo {
   GS_ALGO_PREFILL = 2,  /* tcgen05/TMEM/TMA tensor-core kernel (compute-bound)        */
   GS_ALGO_PREFILL_DENSE = 3  /* tcgen05 kernel over zero-filled 256-row windows: tensor
                                 work of the dense layer, no gather; 1 x 128 and 1 x 256
-                                groups; GS_ALGO_AUTO picks it from T = 17              */
+                                groups; GS_ALGO_AUTO picks it from T = 17, and below
+                                where it is the faster one for the layers of the call  */
 } gs_algo;
 
 typedef struct gs_packed gs_packed;   /* opaque, library-owned */
@@ -137,6 +138,12 @@ gs_status gs_packed_group_shape(const gs_packed* p, int32_t* g_out, int32_t* g_i
  * T      number of tokens; T == 0 is a no-op, T < 0 is INVALID_ARG.
  * y_dev  bf16 [T][out] row-major, caller-owned; fully overwritten (rows of
  *        outputs with no kept group are written as +0.0).
+ * Infinities and NaN in x reach that token's outputs alone.  An output row that
+ * keeps the group of such an input is non-finite, as the products make it.  A
+ * row that prunes it has either the value of its kept groups alone or NaN
+ * (0 x inf): which of the two depends on the kernel, and so on T, the layer and
+ * the other layers of a batch, since most kernels multiply a pruned group by
+ * zero where other rows nearby keep theirs.
  * Errors: INVALID_ARG, UNSUPPORTED (a ninth stream on one handle), OOM (a new
  * stream's scratch), CUDA.  Asynchronous on `stream`.
  */
@@ -148,12 +155,13 @@ gs_status gs_linear_ex(const void* x_dev, const gs_packed* p, int64_t T, void* y
 
 /*
  * gs_linear_batched - n independent layers, ys[i] = xs[i] W_hat_i^T for the
- * i-th handle, all with the same token count T.  In the decode regime all n
- * layers share one launch per 16 tokens (one grid streams every layer's kept
- * groups), or, from 20 M weights in all, up to 8 row-group layers one launch of
- * the zero-filled kernel; in the prefill regime (T >= 17) up to 8 layers share
- * one launch (one list of output tiles).  Results are those of gs_linear for each layer
- * (prefill: bit for bit).  Same per-layer semantics and errors as gs_linear.
+ * i-th handle, all with the same token count T.  Up to 16 tokens all n layers
+ * share one launch of the decode kernel (one grid streams every layer's kept
+ * groups), or up to 8 row-group layers one launch of the zero-filled kernel,
+ * whichever is the faster for these layers; from T = 17 up to 8 layers share
+ * one launch (one list of output tiles).  Results are those of gs_linear for each
+ * layer (from T = 17 bit for bit where x is finite).  Same per-layer semantics and
+ * errors as gs_linear.
  * 1 <= n <= 32 (n == 0 is a no-op); the handles must be distinct.
  */
 gs_status gs_linear_batched(int32_t n, const void* const* xs_dev, const gs_packed* const* ps,
