@@ -367,8 +367,7 @@ static gs_status linear_impl(const void* x_dev, const gs_packed* p, int64_t T, v
         return launch_prefill_dense(&x_dev, &p, 1, T, &y_dev, s, nullptr, true);
       algo = GS_ALGO_DECODE;
     }
-    else if (prefill_prefers_dense(p)) algo = GS_ALGO_PREFILL_DENSE;
-    else algo = p->G <= prefill_max_chunks() ? GS_ALGO_PREFILL : GS_ALGO_DECODE;
+    else algo = p->kept == 0 || prefill_prefers_dense(p) ? GS_ALGO_PREFILL_DENSE : GS_ALGO_DECODE;
   }
   if (algo == GS_ALGO_PREFILL) return launch_prefill(x_dev, p, T, y_dev, s);
   if (algo == GS_ALGO_PREFILL_DENSE) {
@@ -454,31 +453,17 @@ gs_status gs_linear_batched(int32_t n, const void* const* xs_dev, const gs_packe
     }
   }
   if (T >= kPrefillMinTokens) {
-    // layers the prefill kernel takes share batched launches; any other goes alone
-    // (layers the zero-filled kernel runs faster go there, batched the same way)
-    std::vector<const void*> xp, xd;
-    std::vector<const gs_packed*> pp, pd;
-    std::vector<void*> yp, yd;
+    // the zero-filled kernel's layers share launches; any other layer goes alone
+    std::vector<int> idx;
     for (int i = 0; i < n; ++i) {
       if (prefill_prefers_dense(ps[i])) {
-        xd.push_back(xs_dev[i]);
-        pd.push_back(ps[i]);
-        yd.push_back(ys_dev[i]);
-      } else if (ps[i]->G <= prefill_max_chunks()) {
-        xp.push_back(xs_dev[i]);
-        pp.push_back(ps[i]);
-        yp.push_back(ys_dev[i]);
-      } else {
-        const gs_status st = linear_impl(xs_dev[i], ps[i], T, ys_dev[i], stream, GS_ALGO_AUTO);
-        if (st != GS_OK) return st;
+        idx.push_back(i);
+        continue;
       }
-    }
-    if (!pd.empty()) {
-      const gs_status st = launch_prefill_dense(xd.data(), pd.data(), (int)pd.size(), T, yd.data(), s);
+      const gs_status st = linear_impl(xs_dev[i], ps[i], T, ys_dev[i], stream, GS_ALGO_AUTO);
       if (st != GS_OK) return st;
     }
-    if (pp.empty()) return GS_OK;
-    return launch_prefill_batched(xp.data(), pp.data(), (int)pp.size(), T, yp.data(), s);
+    return launch_prefill_dense(xs_dev, ps, (int)idx.size(), T, ys_dev, s, idx.data());
   }
   if (decode_prefers_dense(ps, n, T)) {
     std::vector<int> idx;

@@ -189,9 +189,6 @@ int decode_max_tokens();
 // prefill.cu
 gs_status prefill_prepare_weight_maps(gs_packed* p);
 gs_status launch_prefill(const void* x, const gs_packed* p, int64_t T, void* y, cudaStream_t s);
-gs_status launch_prefill_batched(const void* const* xs, const gs_packed* const* ps, int n, int64_t T,
-                                 void* const* ys, cudaStream_t s);
-int prefill_max_chunks();
 // prefill_dense.cu: zero-filled windows (1 x 128 / 1 x 256 layers with kept groups)
 // (layers ps[idx[k]], k < n, when idx is given; else ps[0..n)).  split: at T <= 16 units may be
 // split along the input, with the decode path's per-stream scratch (1 x KW layers).
