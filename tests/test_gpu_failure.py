@@ -2,7 +2,7 @@
 use of one packed handle from several streams at once.
 
 * A bounded wait that runs out: the test hook makes the first CTA (or CTA
-  pair) of the next decode or prefill launch wait on a library word that
+  pair) of the next few-token or prefill launch wait on a library word that
   nothing ever sets, before it issues any copy or MMA.  The wait runs out,
   the launch records GS_ERR_DEVICE_TIMEOUT, gs_device_status reports it, and
   the next normal call on the same handle must again match the oracle (the
@@ -58,8 +58,11 @@ def test_decode_wait_timeout_then_recovery(gs, T):
     assert gs.device_status() == gs.GS_OK
 
 
-def test_batched_decode_wait_timeout_then_recovery(gs):
-    shapes = [(4096, 11008, 0.5, 51), (11008, 4096, 0.6, 52), (512, 4096, 0.3, 53)]
+# the decode kernel (blocks of several units each), and layers that the zero-filled kernel takes, which
+# the same hook reaches at T <= 16
+@pytest.mark.parametrize("shapes", [[(512, 11008, 0.5, 54), (1024, 8192, 0.6, 55), (256, 4096, 0.3, 56)],
+                                    [(4096, 11008, 0.5, 51), (11008, 4096, 0.6, 52), (512, 4096, 0.3, 53)]])
+def test_batched_decode_wait_timeout_then_recovery(gs, shapes):
     layers = [make(gs, *s) for s in shapes]
     T = 4
     xbs = [wl.random_activation_bits(T, s[1], seed=60 + i) for i, s in enumerate(shapes)]

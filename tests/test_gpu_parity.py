@@ -208,9 +208,10 @@ def test_prefill_dense_large_ragged_layers(gs, go, gi):
 
 
 def test_prefill_more_tiles_than_the_tile_list(gs):
-    """Launches with more tiles than the balanced tile list holds (2048) fall back to the fixed
-    stride: a 41120-row layer on the gathering kernel (8 x 257 tiles) and a 65792-row layer on the
-    zero-filled kernel (8 x 257 units) at T = 2048, sampled tokens against the oracle."""
+    """Launches with more tiles than the balanced tile list holds (2048) take them at a fixed
+    stride, as the gathering kernel always does: a 41120-row layer there (8 x 257 tiles) and a
+    65792-row layer on the zero-filled kernel (8 x 257 units) at T = 2048, sampled tokens against
+    the oracle."""
     T = 2048
     for out, algo, seed in ((41120, gs.ALGO_PREFILL, 65), (65792, gs.ALGO_PREFILL_DENSE, 66)):
         Wb, B = layer(out, 256, 0.5, seed)
@@ -289,7 +290,7 @@ def test_block_workload_decode_batched(gs):
 def test_decode_batched_many_layers(gs, n):
     """More layers in one decode launch than the small parameter block holds
     (up to the 32-layer limit), with mixed shapes and densities, the split and
-    unsplit unit paths, and T = 3 and 16."""
+    unsplit unit paths, and T = 3 and 16.  One launch a call: the decode kernel's."""
     import torch
     outs = [64, 200, 256, 512, 1000, 1024]
     inps = [256, 512, 1024, 2048, 2816]
@@ -305,17 +306,46 @@ def test_decode_batched_many_layers(gs, n):
         xs = [wl.random_activation_bits(T, W.shape[1], seed=700 + 17 * i + T) for i, W in enumerate(Ws)]
         xd = [to_dev(x) for x in xs]
         ys = [torch.empty((T, W.shape[0]), dtype=torch.bfloat16, device="cuda") for W in Ws]
+        before = gs.launch_count()
         gs.linear_batched_into(xd, ps, ys)
+        assert gs.launch_count() - before == 1
         for i in range(n):
             assert_within_bound(to_bits(ys[i]), xs[i], Ws[i], Bs[i], what=f"batched n={n} layer {i} T={T}")
     assert gs.device_status() == gs.GS_OK
 
 
-@pytest.mark.parametrize("n,T", [(3, 200), (11, 300), (7, 1024)])   # T = 1024: the zero-filled kernel
+@pytest.mark.parametrize("gi", [256, 128])
+def test_zero_filled_few_tokens_many_layers(gs, gi):
+    """More than eight layers at few tokens on the zero-filled kernel: two launches, the second for
+    one or two layers, with ragged rows and a layer without kept groups between."""
+    import torch
+    outs = [18001, 20000, 16385, 17664, 19000, 18432, 20481, 16400, 17001, 18500]
+    inps = [512 if gi == 256 else 384, 256, 256, 512, 256, 256, 256, 256, 256, 256]
+    dens = [0.3, 0.5, 0.9, 0.05, 0.5, 0.0, 0.7, 0.5, 0.2, 1.0]
+    Ws, Bs, ps = [], [], []
+    for i, (out, inp, d) in enumerate(zip(outs, inps, dens)):
+        Wb = wl.random_weight_bits(out, inp, seed=1200 + i)
+        B = wl.random_mask(out, inp // gi, d, seed=1300 + i)
+        Ws.append(Wb)
+        Bs.append(B)
+        ps.append(gs.pack_groups(to_dev(Wb), torch.from_numpy(np.ascontiguousarray(B, dtype=np.uint8)).cuda(), 1, gi))
+    for T in (9, 16):
+        xs = [wl.random_activation_bits(T, inp, seed=1400 + 31 * i + T) for i, inp in enumerate(inps)]
+        ys = [torch.full((T, out), 7.0, dtype=torch.bfloat16, device="cuda") for out in outs]
+        before = gs.launch_count()
+        gs.linear_batched_into([to_dev(x) for x in xs], ps, ys)
+        assert gs.launch_count() - before == 2
+        for i in range(len(outs)):
+            yr, A = orc.linear(xs[i], Ws[i], Bs[i], 1, gi)
+            assert np.all(np.abs(to_f64(ys[i]) - yr) <= 2.0 ** -7 * A + 1e-6), (i, T)
+    assert gs.device_status() == gs.GS_OK
+
+
+@pytest.mark.parametrize("n,T", [(3, 200), (11, 300), (7, 1024)])
 def test_prefill_batched_matches_single(gs, n, T):
     """A batched prefill call (several layers with one T share launches of up
-    to 8 layers) gives bit for bit the single-layer results and stays within
-    the bound; layers without kept groups give zeros."""
+    to 8 layers of the zero-filled kernel) gives bit for bit the single-layer
+    results and stays within the bound; layers without kept groups give zeros."""
     import torch
     shapes = [(4096, 4096, 0.5), (1000, 1024, 0.3), (512, 2816, 0.8), (300, 256, 0.0), (2048, 512, 1.0),
               (160, 768, 0.5), (1100, 2048, 0.05)]
