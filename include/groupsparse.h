@@ -354,9 +354,10 @@ gs_status gs_gumbel_select(const float* logits_dev, const float* noise_dev, int6
  *     dL/dB[u][v] = sum over the cells (r, k) of group (u, v) of W[r][k] dL/dW_hat[r][k]
  *     dL/dl[u][v] = dL/dB[u][v] ds/dl[u][v]             (the estimator)
  *     dL/dx = dy W_hat
- * Every group receives a logit gradient, pruned ones included.  The two
- * products are dense GEMMs done by cuBLAS (fp32 accumulation); the group
- * reduction and the estimator are a kernel of this library.
+ * Every group receives a logit gradient, pruned ones included.  For 1 x 128 and
+ * 1 x 256 groups and out a multiple of 64, dL/dl is one kernel of this library
+ * that keeps dL/dW_hat on chip (fp32); elsewhere dL/dW_hat is a dense GEMM done
+ * by cuBLAS (fp32) and a second kernel reduces it.  dL/dx is a cuBLAS GEMM.
  *
  * x_dev       bf16 [T][in] (the forward input).      W_dev  bf16 [out][in] (dense, frozen).
  * p           handle of W packed with the sampled mask B (any supported group shape).
@@ -365,7 +366,8 @@ gs_status gs_gumbel_select(const float* logits_dev, const float* noise_dev, int6
  * dlogits_dev float32 [out/g_out][in/g_in], overwritten.
  * dx_dev      bf16 [T][in], overwritten, or NULL (no input gradient).
  * workspace   device scratch of gs_masked_linear_backward_workspace bytes
- *             (16-byte aligned; it holds dL/dW_hat and, with dx, W_hat).
+ *             (16-byte aligned; room for dL/dW_hat, which the one-kernel form
+ *             leaves untouched, and, with dx, for W_hat).
  * Not for use inside a CUDA graph capture (cuBLAS may allocate on first use).
  * Errors: INVALID_ARG (nulls, sizes, alignment, workspace too small), CUDA.
  */

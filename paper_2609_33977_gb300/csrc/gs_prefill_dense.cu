@@ -18,8 +18,9 @@
 // rows only, and nothing is written there by threads, so no generic-to-async
 // proxy fence lies between the weights and the tensor cores.  (With the rows
 // placed in shared memory by cp.async, as zero-filled B operands, the copies'
-// fences and the second operand's bytes held a 7B block at T = 2048 to 547 us,
-// 1.52 PFLOP/s dense-equivalent; now 405 us, 2.05 PFLOP/s, at the chip's power limit.)
+// fences and the second operand's bytes held a 7B block at T = 2048 to 576 us,
+// 1.44 PFLOP/s dense-equivalent; now 478 us, 1.73 PFLOP/s, a library GEMM's sustained
+// rate at the chip's power limit.)
 //
 // What bounds it.  At N = 256 the tensor cores.  At small N the stream of kept weights
 // (5.7 TB/s) and, where units are few, the chain of hand-offs of a stage (copy ->
@@ -59,7 +60,7 @@ constexpr int kDConvWarp0 = 4, kDConvSets = 2, kDConvWarps = 4 * kDConvSets;   /
 constexpr int kDEpiWarp0 = kDConvWarp0 + kDConvWarps, kDEpiWarps = 8;
 constexpr int kDThreads = (kDEpiWarp0 + kDEpiWarps) * 32;
 constexpr int kDMmaWarp = 2;
-constexpr uint32_t kDTmemCols = 512;              // D first, then the A slots of 64 columns each
+constexpr uint32_t kDTmemCols = 512;              // D first, then the A slots of SK / 2 columns each
 constexpr int kDMaxLayers = 8;
 constexpr int kDMaxChunks = 32767;                // wider inputs stay on the other kernels
 constexpr int kDWMaps = 8;                        // W box heights: 16, 32, ..., 128 rows (square: g, 2g, ..., 128)
@@ -1022,7 +1023,7 @@ cudaError_t d_launch(const cudaLaunchConfig_t& cfg, const DParams& P) {
 
 // Parts per window of each layer of a launch of at most 16 tokens.  Whole windows
 // alone can be too few or too long to fill 76 CTA pairs: a 5120 x 13824 layer (20
-// windows of 54 items) took 35 us, 21 in three parts.  But a part costs what about
+// windows of 54 items) took 35 us, 19 in three parts.  But a part costs what about
 // six items do (partial sums out and in, an atomic): 13824 x 5120 took 17 us whole
 // and 21 to 30 us in four parts, a 7B block 37 us whole and 43 us with its 43-item
 // windows in parts of ten.

@@ -13,11 +13,12 @@
 //             W (.) dL/dW_hat, and the STE gives dL/dl = dL/dB ds/dl;
 //             dL/dx = dy W_hat.
 //
-// The two products of the backward are plain dense GEMMs (dy^T x over all
-// groups, pruned ones included, since the STE passes gradients to every
-// selector; dy W_hat on the masked weight) and go to cuBLAS.  The group
-// reduction with the STE factor and the sampling are kernels of this file; the
-// forward pass is gs_pack with the sampled mask followed by gs_linear.
+// dy^T x covers all groups, pruned ones included, since the STE passes gradients
+// to every selector.  For row groups with whole 64-row slabs it stays on chip
+// (gs_group_grad.cu); elsewhere cuBLAS forms it as a plain dense GEMM in the
+// workspace and a kernel of this file reduces it with the STE factor.  dy W_hat
+// on the masked weight is a cuBLAS GEMM.  The sampling is a kernel of this file;
+// the forward pass is gs_pack with the sampled mask followed by gs_linear.
 #include "gs_common.cuh"
 
 #include <cublas_v2.h>

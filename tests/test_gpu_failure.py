@@ -129,6 +129,7 @@ def test_failed_allocation_returns_oom_and_frees_everything(gs):
     W = to_dev(Wb)
     mask = torch.from_numpy(B).cuda()
     gs.pack(W, mask).free()            # warm-up: the library's per-device flag exists from here on
+    gs.trim()                          # nothing idle: what comes back below comes back to the device
     torch.cuda.synchronize()
     free0 = torch.cuda.mem_get_info()[0]
     failures = 0
@@ -139,6 +140,7 @@ def test_failed_allocation_returns_oom_and_frees_everything(gs):
         except gs.GroupSparseError as e:
             assert e.status == gs.GS_ERR_OOM, e
             failures += 1
+            gs.trim()
             torch.cuda.synchronize()
             assert torch.cuda.mem_get_info()[0] == free0, f"allocation {nth}: bytes not given back"
             continue
@@ -151,6 +153,7 @@ def test_failed_allocation_returns_oom_and_frees_everything(gs):
         p.free()
         break
     assert failures >= 6                # every buffer gs_pack allocates was made to fail once
+    gs.trim()
     torch.cuda.synchronize()
     assert torch.cuda.mem_get_info()[0] == free0
 
